@@ -183,7 +183,8 @@ CUBIC_API cubic_status_t cubic_rl_plan_set_wait_limit(cubic_rl_plan_t plan, uint
 
 /* Test support for the failure path of the bounded waits (no counterpart in the paper).
  * Arms a one-shot setting for the whole process: the next Y-pass launch that uses a
- * TMA-pipelined launch shape -- on any plan, or inside cubic_rl_deconvolve_noalloc -- waits
+ * TMA-pipelined launch shape -- on any plan, or inside cubic_rl_deconvolve_noalloc, which
+ * takes the pass-by-pass form while the setting is armed -- waits
  * at most wait_ns per tile, and its first CTA does not issue the copy of its first tile.
  * That CTA's wait then runs out: it sets the device error word, waits for the copies it
  * did issue and returns, so no copy is left in flight and the context stays usable.  The

@@ -15,10 +15,11 @@
 #include <map>
 #include <mutex>
 #include <new>
+#include <tuple>
 #include <vector>
 
 #include "../../include/cubic_rl.h"
-#include "lens.cuh"
+#include "plane.cuh"
 #include "registry.cuh"
 
 using namespace cubic;
@@ -261,6 +262,23 @@ struct cubic_rl_plan_s {
     bool allow_real_h = false;  // set by cubic_rl_plan (may allocate Hr)
     bool use_real_h = false;
     float *Hr = nullptr;        // [nz][ny][xp], owned
+    // the fused form (plane.cuh): fuse.ok where it serves this plan; HF / HFr are H in its
+    // layout (owned, or H itself where own_hf is false); pinned: the caller chose launch
+    // shapes or chunks of the pass-by-pass form, which plain calls then take
+    struct Fused {
+        bool ok = false;
+        PlaneGeo g;
+        int threads = 0;              // threads per plane CTA, single-volume launches
+        int64_t conv_blocks = 0;
+        size_t conv_smem = 0;
+        size_t tab_elems = 0;         // the constant block, float2
+        bool c_is_z = false;
+    } fuse;
+    float2 *ftab = nullptr;           // the fused form's constants (plane_tables), owned
+    bool pinned = false;
+    float2 *HF = nullptr;
+    float *HFr = nullptr;
+    bool own_hf = false;
     // linear ("same"-mode) boundaries: nz, ny, nx are then the transform's dims, the image is
     // iz x iy x ix (V, rows count its voxels and rows), the plan keeps the image and the
     // estimate in rows zero-padded to nx (lin: [2][iz][iy][nx]) and the spectrum work array
@@ -347,15 +365,163 @@ static cudaError_t counted(cubic_rl_plan_s *p, int kind, cudaStream_t st, F &&la
 
 static const int kXKind[XM_COUNT] = {KK_X_FWD, KK_X_INV, KK_X_RATIO, KK_X_UPDATE, KK_X_FINAL};
 
-static cudaError_t run_x(cubic_rl_plan_s *p, int mode, const XArgs &a, cudaStream_t st)
+// ------------------------------------------------------------------ the fused form
+
+static bool use_fused(const cubic_rl_plan_s *p) { return p->fuse.ok && !p->pinned; }
+
+// Largest plane that takes the fused form
+constexpr int64_t kFuseSmem = 122 * 1024;
+
+// Most threads a plane CTA of `smem` bytes can have when `want` of them share an SM
+static int plane_cta_threads(size_t smem, int64_t want)
+{
+    int64_t k = (int64_t)(kPlaneSmemMax / (smem + 1024));
+    k = std::max<int64_t>(1, std::min(k, want));
+    return std::max(64, kPlaneThreads / (int)k / 32 * 32);
+}
+
+// Geometry of the fused form with c = z (planes along y) or c = y (planes along z); false
+// where the lengths or the plane's size rule it out.
+static bool fuse_geometry(const cubic_rl_plan_s *p, bool c_is_z, cubic_rl_plan_s::Fused *f)
+{
+    const int64_t nc = c_is_z ? p->nz : p->ny, np = c_is_z ? p->ny : p->nz;
+    const PlaneLen x = plane_len(PlaneX{}, p->nx), c = plane_len(PlaneC{}, nc), v = plane_len(ConvLens{}, np);
+    if (x.r1 == 0 || c.r1 == 0 || v.r1 == 0) return false;
+    PlaneGeo g;
+    g.nx = (int)p->nx;
+    g.nc = (int)nc;
+    g.np = (int)np;
+    g.lines = (int)((p->nx + 1) / 2);
+    // slots of a pair line and, for odd nx, a spare one.  A pitch of 4 mod 16 slots puts the
+    // rows that four adjacent columns' threads touch in different banks; 4 spare slots after
+    // every r1 pair lines (r1 even) do so for the second stage's strided rows.
+    g.xs = (x.slots + (int)(p->nx % 2) + 11) / 16 * 16 + 4;
+    g.cr1 = c.r1;
+    g.bs = c.r1 * g.xs + (c.r1 % 2 == 0 ? 4 : 0);
+    g.off_twc = (x.tw + 1) / 2 * 2;
+    g.off_tab = g.off_twc + (c.tw + 1) / 2 * 2;
+    g.off_neg = g.off_tab + (g.lines + 3) / 4 * 2;
+    g.off_plane = g.off_neg + (g.nc + 3) / 4 * 2;
+    const int last = (g.nc + 1) / 2 - 1;  // pair lines 0 .. last
+    const int64_t slots = (int64_t)(last / c.r1) * g.bs + (int64_t)(last % c.r1 + 1) * g.xs;
+    const int64_t smem = ((int64_t)g.off_plane + slots) * (int64_t)sizeof(float2);
+    if (smem > kFuseSmem) return false;
+    g.smem = (int)smem;
+    g.mv = g.lines * g.nc + (p->nx % 2 == 0 ? g.nc : 0);
+    g.m = (g.mv + 15) / 16 * 16;
+    g.rs = (int)(c_is_z ? p->ny * p->nx : p->nx);
+    g.ps = (int)(c_is_z ? p->nx : p->ny * p->nx);
+    f->ok = true;
+    f->g = g;
+    f->c_is_z = c_is_z;
+    f->tab_elems = (size_t)g.off_plane + (size_t)v.tw;
+    f->conv_blocks = conv_blocks_of(v, g.mv);
+    f->conv_smem = conv_smem_of(ConvLens{}, np);
+    // Warps per CTA: the fewest that run the fewest rounds of x and c tasks (weighted by a
+    // task's passes over its lanes), at most 12 where the planes are small enough that four
+    // share an SM: two CTAs then fit its registers, so other streams' volumes can run beside
+    // this one's (16 differentiable 128x128x64 volumes over 4 streams: 47 ms with 16 warps, 34
+    // with 12; a single one loses 3 us of 38).
+    auto task_cost = [](const PlaneLen &l, int w) { return (w * l.r1 + 31) / 32 * l.r0 + (w * l.r0 + 31) / 32 * l.r1; };
+    const int tc = (g.lines + c.col_lines - 1) / c.col_lines, tr = (last + x.row_lines) / x.row_lines;
+    const int cc = task_cost(c, c.col_lines), cr = task_cost(x, x.row_lines);
+    const int most = std::min(g.smem <= 55 * 1024 ? 12 : 24, plane_cta_threads(g.smem, (np + 151) / 152) / 32);
+    int best = 1;
+    int64_t best_cost = INT64_MAX;
+    for (int w = 1; w <= most; ++w) {
+        const int64_t cost = (int64_t)((tc + w - 1) / w) * cc + (int64_t)((tr + w - 1) / w) * cr * 5 / 4;
+        if (cost < best_cost) {
+            best_cost = cost;
+            best = w;
+        }
+    }
+    f->threads = 32 * best;
+    return true;
+}
+
+static void fuse_setup(cubic_rl_plan_s *p)
+{
+    p->fuse = cubic_rl_plan_s::Fused();
+    if (p->linear) return;
+    cubic_rl_plan_s::Fused z, y;
+    const bool hz = fuse_geometry(p, true, &z), hy = fuse_geometry(p, false, &y);
+    // the smaller plane (more CTAs, and more of them on an SM), but an even c axis before an odd
+    // one, which takes two more passes over the plane (81x150x135 voxels: 69 us an iteration
+    // with c = 150, 87 us with c = 81)
+    auto cost = [](const cubic_rl_plan_s::Fused &f) { return f.g.nc + (f.g.nc % 2 ? 1024 : 0); };
+    if (hz && (!hy || cost(z) <= cost(y))) p->fuse = z;
+    else if (hy) p->fuse = y;
+}
+
+// the plan's constant block, from its twiddle tables
+__global__ void __launch_bounds__(256) k_plane_tables(PlaneGeo g, float2 *tab, const float2 *wx, const float2 *wc,
+                                                      const float2 *wp)
+{
+    plane_tables(g, tab, wx, wc, wp);
+}
+
+static cudaError_t launch_plane_tables(const cubic_rl_plan_s *p, cudaStream_t st)
+{
+    const bool z = p->fuse.c_is_z;
+    k_plane_tables<<<1, 256, 0, st>>>(p->fuse.g, p->ftab, p->tw_x, z ? p->tw_z : p->tw_y,
+                                      z ? p->tw_y : p->tw_z);
+    return cudaGetLastError();
+}
+
+static PlaneArgs plane_args(const cubic_rl_plan_s *p, const XArgs &x)
+{
+    PlaneArgs a;
+    a.x = x;
+    a.tab = reinterpret_cast<const float4 *>(p->ftab);
+    a.g = p->fuse.g;
+    return a;
+}
+
+static ConvArgs conv_args(const cubic_rl_plan_s *p, float2 *spec)
+{
+    ConvArgs a{};
+    a.spec = spec;
+    a.H = p->HF;
+    a.Hr = p->use_real_h ? p->HFr : nullptr;
+    a.tw = p->ftab + p->fuse.g.off_plane;
+    a.m = p->fuse.g.m;
+    a.mv = p->fuse.g.mv;
+    a.n = p->fuse.g.np;
+    a.scale = 1.f;
+    return a;
+}
+
+static cudaError_t launch_plane_plan(const cubic_rl_plan_s *p, int mode, const XArgs &a, cudaStream_t st)
+{
+    const cubic_rl_plan_s::Fused &f = p->fuse;
+    return launch_plane(mode, plane_args(p, a), nullptr, f.g.np, f.threads, (size_t)f.g.smem, st);
+}
+
+static cudaError_t launch_conv_plan(const cubic_rl_plan_s *p, const ConvArgs &a, int mode, cudaStream_t st)
+{
+    return launch_conv(a, nullptr, p->fuse.conv_blocks, mode, p->fuse.conv_smem, st);
+}
+
+// ------------------------------------------------------------------ running the passes
+
+// the x pass of the pass-by-pass form
+static cudaError_t run_x_pass(cubic_rl_plan_s *p, int mode, const XArgs &a, cudaStream_t st)
 {
     return counted(p, kXKind[mode], st, [&] { return p->kx->xv[p->vx].fn[mode](a, st); });
 }
 
-// an X pass counted under another kind (the accelerated-RL forms of XM_FWD / XM_FINAL)
+// an X pass counted under another kind (the accelerated-RL forms of XM_FWD / XM_FINAL); in
+// the fused form the plane kernel of that mode
 static cudaError_t run_x_as(cubic_rl_plan_s *p, int mode, int kind, const XArgs &a, double bytes, cudaStream_t st)
 {
-    return counted(p, kind, st, [&] { return p->kx->xv[p->vx].fn[mode](a, st); }, bytes);
+    return counted(p, kind, st, [&] {
+        return use_fused(p) ? launch_plane_plan(p, mode, a, st) : p->kx->xv[p->vx].fn[mode](a, st);
+    }, bytes);
+}
+
+static cudaError_t run_x(cubic_rl_plan_s *p, int mode, const XArgs &a, cudaStream_t st)
+{
+    return run_x_as(p, mode, kXKind[mode], a, -1.0, st);
 }
 
 // Failure-path test (cubic_test_skip_next_tile_copy): armed with a wait limit, the next
@@ -429,6 +595,15 @@ static XArgs x_args(const cubic_rl_plan_s *p, bool full = false)
     return a;
 }
 
+// A plain iteration in the fused form takes 1 off the ratio before its transform and adds
+// the PSF's sum back to the correlation (XArgs::h0).  H carries 1 / 2V there.  Not in the
+// differentiable path, which needs the spectrum of the ratio itself.
+static void center_ratio(const cubic_rl_plan_s *p, XArgs &a)
+{
+    a.h0 = p->HF;
+    a.h0_scale = (float)(2.0 * (double)p->V);
+}
+
 // Forward 3D real-to-half-complex transform of `real` into `spec`, optionally
 // scaled (scale applies in the Z pass).
 static cubic_status_t enqueue_forward3(cubic_rl_plan_s *p, const float *real, float2 *spec, float scale,
@@ -437,10 +612,19 @@ static cubic_status_t enqueue_forward3(cubic_rl_plan_s *p, const float *real, fl
     XArgs xa = x_args(p, full);
     xa.spec_out = spec;
     xa.src = real;
-    CUBIC_CUDA(run_x(p, XM_FWD, xa, st));
+    CUBIC_CUDA(run_x_pass(p, XM_FWD, xa, st));
     CUBIC_CUDA(run_y(p, y_args(p, spec, 0, 0, p->xh, full), st));
     CUBIC_CUDA(run_z(p, z_args(p, spec, ZM_FWD_SCALE, scale, 0, p->xh, full), st));
     return CUBIC_OK;
+}
+
+// the fused form's convolution kernel, counted as the z product
+static cudaError_t run_conv(cubic_rl_plan_s *p, const ConvArgs &a, int zmode, cudaStream_t st)
+{
+    const int mode = conv_mode(p, zmode);
+    const double arrays = mode == ZM_MUL_REAL ? 2.5 : 3.0;
+    return counted(p, mode == ZM_CORR ? KK_Z_CORR : KK_Z_CONV, st, [&] { return launch_conv_plan(p, a, zmode, st); },
+                   arrays * 8.0 * (double)p->rows * (double)p->xh);
 }
 
 // Y forward, Z (product with H or conj H), Y inverse on the plan's spectrum.
@@ -450,6 +634,10 @@ static cubic_status_t enqueue_forward3(cubic_rl_plan_s *p, const float *real, fl
 // write of the spectrum (plus H) instead of three of each.
 static cubic_status_t enqueue_yzy(cubic_rl_plan_s *p, float2 *spec, int zmode, cudaStream_t st)
 {
+    if (use_fused(p)) {
+        CUBIC_CUDA(run_conv(p, conv_args(p, spec), zmode, st));
+        return CUBIC_OK;
+    }
     const int64_t step = p->chunk > 0 ? p->chunk : p->xh;
     for (int64_t c0 = 0; c0 < p->xh; c0 += step) {
         const int64_t c1 = c0 + step < p->xh ? c0 + step : p->xh;
@@ -500,6 +688,45 @@ __global__ void k_place_psf(const float *__restrict__ psf, int64_t kz, int64_t k
     }
 }
 
+// Hr = Re src, and H = Re src (imaginary parts dropped): the fused form's real H
+__global__ void k_real_part(const float2 *__restrict__ src, float2 *__restrict__ H, float *__restrict__ Hr, int64_t n)
+{
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const float h = src[i].x;
+        Hr[i] = h;
+        H[i] = make_float2(h, 0.f);
+    }
+}
+
+// H in the fused form's layout, from h0 in the work array: h0 -> spectrum (in HF) -> the
+// work array -> HF.  The plane kernel's forward c transform leaves its spectrum doubled
+// (here and in every convolution), so the scale is 1 / 4V.
+static cubic_status_t load_fused_h(cubic_rl_plan_s *p, const float *h0, bool even, cudaStream_t st)
+{
+    const int64_t n = (int64_t)p->fuse.g.np * p->fuse.g.mv;
+    XArgs xa = x_args(p);
+    xa.src = h0;
+    xa.spec_out = p->HF;
+    CUBIC_CUDA(counted(p, KK_X_FWD, st, [&] { return launch_plane_plan(p, XM_FWD, xa, st); }));
+    ConvArgs ca = conv_args(p, p->HF);
+    ca.Hr = nullptr;
+    ca.out = p->ws;
+    ca.scale = (float)(1.0 / (4.0 * (double)p->V));
+    CUBIC_CUDA(counted(p, KK_Z_FWD, st, [&] { return launch_conv_plan(p, ca, ZM_FWD_SCALE, st); }));
+    if (!even) {
+        CUBIC_CUDA(cudaMemcpyAsync(p->HF, p->ws, (size_t)n * sizeof(float2), cudaMemcpyDeviceToDevice, st));
+        return CUBIC_OK;
+    }
+    if (!p->HFr) {
+        void *m = nullptr;
+        CUBIC_CUDA(cudaMalloc(&m, (size_t)n * sizeof(float)));
+        p->HFr = (float *)m;
+    }
+    k_real_part<<<grid_for(n, 256), 256, 0, st>>>(p->ws, p->HF, p->HFr, n);
+    CUBIC_CUDA(cudaGetLastError());
+    return CUBIC_OK;
+}
+
 static cubic_status_t load_psf(cubic_rl_plan_s *p, const float *psf, cudaStream_t st)
 {
     cubic_status_t s = ensure_workspace(p);
@@ -536,9 +763,11 @@ static cubic_status_t load_psf(cubic_rl_plan_s *p, const float *psf, cudaStream_
         even = host == 0;
     }
     p->use_real_h = false;  // H itself is complex while it is computed
-    s = enqueue_forward3(p, h0, p->H, (float)(1.0 / (double)Vt), st, true);
+    if (p->HF != p->H) s = enqueue_forward3(p, h0, p->H, (float)(1.0 / (double)Vt), st, true);
     if (p->linear) CUBIC_CUDA(cudaFreeAsync(h0, st));
-    if (s != CUBIC_OK || !even) return s;
+    if (s != CUBIC_OK) return s;
+    if (p->fuse.ok && (s = load_fused_h(p, h0, even, st)) != CUBIC_OK) return s;
+    if (!even) return s;
     if (!p->Hr) {
         void *m = nullptr;
         CUBIC_CUDA(cudaMalloc(&m, h_elems(p) * sizeof(float)));
@@ -630,6 +859,16 @@ static cubic_status_t plan_build(cubic_rl_plan_s *p, const float *psf, cudaStrea
     e = cudaMalloc(&mem, h_elems(p) * sizeof(float2));
     if (e != cudaSuccess) return bail(fail(CUBIC_ERR_OUT_OF_MEMORY, "H: %s", cudaGetErrorString(e)));
     p->H = (float2 *)mem;
+    fuse_setup(p);
+    if (p->fuse.ok) {
+        e = cudaMalloc(&mem, (size_t)p->fuse.g.np * p->fuse.g.m * sizeof(float2));
+        if (e != cudaSuccess) return bail(fail(CUBIC_ERR_OUT_OF_MEMORY, "H (fused): %s", cudaGetErrorString(e)));
+        p->HF = (float2 *)mem;
+        p->own_hf = true;
+        e = cudaMalloc(&mem, p->fuse.tab_elems * sizeof(float2));
+        if (e != cudaSuccess) return bail(fail(CUBIC_ERR_OUT_OF_MEMORY, "constants (fused): %s", cudaGetErrorString(e)));
+        p->ftab = (float2 *)mem;
+    }
     const int64_t ntw = p->nx + p->ny + p->nz;
     e = cudaMalloc(&mem, ntw * sizeof(float2));
     if (e != cudaSuccess) return bail(fail(CUBIC_ERR_OUT_OF_MEMORY, "twiddles: %s", cudaGetErrorString(e)));
@@ -656,6 +895,7 @@ static cubic_status_t plan_build(cubic_rl_plan_s *p, const float *psf, cudaStrea
     k_twiddles<<<grid_for(p->ny, 128, 1 << 20), 128, 0, st>>>(p->tw_y, (int)p->ny);
     k_twiddles<<<grid_for(p->nz, 128, 1 << 20), 128, 0, st>>>(p->tw_z, (int)p->nz);
     e = cudaGetLastError();
+    if (e == cudaSuccess && p->fuse.ok) e = launch_plane_tables(p, st);
     if (e != cudaSuccess) return bail(fail(CUBIC_ERR_CUDA, "twiddles: %s", cudaGetErrorString(e)));
     s = load_psf(p, psf, st);
     if (s != CUBIC_OK) return bail(s);
@@ -760,6 +1000,11 @@ extern "C" cubic_status_t cubic_rl_plan_destroy(cubic_rl_plan_t plan)
     cudaFree(plan->stage_out);
     cudaFree(plan->bwd);
     cudaFree(plan->Hr);
+    if (plan->own_hf) {
+        cudaFree(plan->HF);
+        cudaFree(plan->ftab);
+    }
+    cudaFree(plan->HFr);
     cudaFree(plan->ws2);
     cudaFree(plan->fsc_sums);
     cudaFree(plan->auto_stats);
@@ -953,6 +1198,7 @@ static cubic_status_t enqueue_rl(cubic_rl_plan_s *p, const float *image, int n_i
     xa.dst = out;
     xa.d = image;
     xa.eps = eps;
+    if (use_fused(p)) center_ratio(p, xa);
     CUBIC_CUDA(run_x(p, XM_FWD, xa, st));  // spectrum of u0
     cubic_status_t s;
     for (int k = 0; k < n_iter; ++k) {
@@ -1033,7 +1279,7 @@ extern "C" cubic_status_t cubic_rl_fft3_inverse(cubic_rl_plan_t plan, void *spec
     XArgs xa = x_args(plan);
     xa.spec_in = sp;
     xa.dst = out;
-    CUBIC_CUDA(run_x(plan, XM_INV, xa, st));
+    CUBIC_CUDA(run_x_pass(plan, XM_INV, xa, st));
     return CUBIC_OK;
 }
 
@@ -1210,6 +1456,7 @@ extern "C" cubic_status_t cubic_rl_plan_set_variants(cubic_rl_plan_t plan, int v
     plan->vx = vx;
     plan->vy = vy;
     plan->vz = vz;
+    plan->pinned = true;
     return CUBIC_OK;
 }
 
@@ -1218,6 +1465,7 @@ extern "C" cubic_status_t cubic_rl_plan_set_chunk(cubic_rl_plan_t plan, int64_t 
     if (!plan) return fail(CUBIC_ERR_INVALID_ARG, "plan must be non-null");
     if (columns < 0 || columns % 16 != 0) return fail(CUBIC_ERR_INVALID_ARG, "chunk must be a multiple of 16 (0: off)");
     plan->chunk = columns;
+    if (columns > 0) plan->pinned = true;
     return CUBIC_OK;
 }
 
@@ -1290,8 +1538,8 @@ extern "C" cubic_status_t cubic_rl_autotune(cubic_rl_plan_t plan, const float *i
         xa.d = img_w;
         xa.eps = 1.f;
         s = time_best(st, prepare, [&]() -> cubic_status_t {
-            CUBIC_CUDA(run_x(plan, XM_RATIO, xa, st));
-            CUBIC_CUDA(run_x(plan, XM_UPDATE, xa, st));
+            CUBIC_CUDA(run_x_pass(plan, XM_RATIO, xa, st));
+            CUBIC_CUDA(run_x_pass(plan, XM_UPDATE, xa, st));
             return CUBIC_OK;
         }, &ms);
         if (ms < best) { best = ms; bx = v; }
@@ -1434,6 +1682,19 @@ __global__ void k_origin_to_center(const float *__restrict__ h0, float *__restri
 // Unnormalised (scale = 1) or normalised (scale = 1/V) inverse 3D transform of a half spectrum.
 static cubic_status_t enqueue_inverse3(cubic_rl_plan_s *p, float2 *spec, float *out, float scale, cudaStream_t st)
 {
+    if (use_fused(p)) {
+        // spec holds a product of two doubled spectra, in native order
+        ConvArgs ca = conv_args(p, p->ws);
+        ca.Hr = nullptr;
+        ca.out = spec;
+        ca.scale = 0.25f * scale;
+        CUBIC_CUDA(counted(p, KK_Z_INV, st, [&] { return launch_conv_plan(p, ca, ZM_INV_SCALE, st); }));
+        XArgs xi = x_args(p);
+        xi.spec_in = p->ws;
+        xi.dst = out;
+        CUBIC_CUDA(run_x(p, XM_INV, xi, st));
+        return CUBIC_OK;
+    }
     CUBIC_CUDA(run_z(p, z_args(p, spec, ZM_INV_SCALE, scale, 0, p->xh), st));
     CUBIC_CUDA(run_y(p, y_args(p, spec, 1, 0, p->xh), st));
     XArgs xa = x_args(p);
@@ -1464,6 +1725,15 @@ static cudaError_t run_z_plain(cubic_rl_plan_s *p, const ZArgs &a, cudaStream_t 
 static cubic_status_t enqueue_yzy_grad(cubic_rl_plan_s *p, float2 *spec, int zmode, float2 *save, float2 *gacc,
                                        const float2 *other, int gconj, cudaStream_t st)
 {
+    if (use_fused(p)) {
+        ConvArgs ca = conv_args(p, spec);
+        ca.save = save;
+        ca.gacc = gacc;
+        ca.gother = other;
+        ca.gconj = gconj;
+        CUBIC_CUDA(run_conv(p, ca, zmode, st));
+        return CUBIC_OK;
+    }
     CUBIC_CUDA(run_y(p, y_args(p, spec, 0, 0, p->xh), st));
     ZArgs za = z_args(p, spec, zmode, 1.f, 0, p->xh);
     za.save = save;
@@ -1632,7 +1902,9 @@ extern "C" cubic_status_t cubic_rl_backward(cubic_rl_plan_t plan, const float *i
         xa.eps = eps;
         const double real = (double)V * 4.0, cplx = (double)p->rows * p->xh * 8.0;
         auto adj = [&](int mode, const XArgs &a, double bytes) {
-            return counted(p, KK_X_ADJOINT, st, [&] { return p->kx->adj[mode - XM_ADJ_R](a, st); }, bytes);
+            return counted(p, KK_X_ADJOINT, st, [&] {
+                return use_fused(p) ? launch_plane_plan(p, mode, a, st) : p->kx->adj[mode - XM_ADJ_R](a, st);
+            }, bytes);
         };
         XArgs au = xa;
         au.adj_w = g;
@@ -1866,6 +2138,7 @@ extern "C" cubic_status_t cubic_rl_deconvolve_auto(cubic_rl_plan_t plan, const f
     xa.dst = uw;
     xa.d = dw;
     xa.eps = eps;
+    if (use_fused(p)) center_ratio(p, xa);
     CUBIC_CUDA(run_x(p, XM_FWD, xa, st));
     int k = 0;
     while (k < max_iter) {
@@ -2013,12 +2286,13 @@ extern "C" cubic_status_t cubic_rl_deconvolve_accel(cubic_rl_plan_t plan, const 
 
     const double spec = (double)p->rows * p->xh * 8.0, real = (double)p->V * 4.0;
     const int64_t L = p->kx->xv[p->vx].L;
-    const int64_t nblocks = (p->rows + 2 * L - 1) / (2 * L);
+    const int64_t nblocks = use_fused(p) ? p->fuse.g.np : (p->rows + 2 * L - 1) / (2 * L);
     XArgs xa = x_args(p);
     xa.spec_in = p->ws;
     xa.spec_out = p->ws;
     xa.d = dw;
     xa.eps = eps;
+    if (use_fused(p)) center_ratio(p, xa);
     xa.src = y;
     CUBIC_CUDA(run_x(p, XM_FWD, xa, st));  // spectrum of y_0
     for (int k = 0; k < n_iter; ++k) {
@@ -2266,6 +2540,7 @@ extern "C" cubic_status_t cubic_rl_deconvolve_monitor(cubic_rl_plan_t plan, cons
     xa.dst = uw;
     xa.d = dw;
     xa.eps = eps;
+    if (use_fused(p)) center_ratio(p, xa);
     CUBIC_CUDA(run_x(p, XM_FWD, xa, st));
     std::vector<float> hrec;
     std::vector<double> hist;  // [k][3]
@@ -2481,13 +2756,13 @@ extern "C" cubic_status_t cubic_fsc_split(cubic_rl_plan_t half_plan, const float
 
 // ------------------------------------------------------------------ batched deconvolution
 //
-// Many volumes of different sizes in one CUDA graph.  For every pass, the volumes whose
-// axis along that pass has a length of one of the all-lengths classes (lens.cuh) share
-// one launch per class, whatever their lengths; the volumes of other lengths share one
-// launch per length (k_*pass with a MultiTable).  A launch's blocks are the
+// Many volumes of different sizes in one CUDA graph.  The volumes that the fused form serves
+// share its launches: the planes of all volumes of one size group in one launch per half
+// iteration, the p-axis convolutions of all of them in another.  The others share one launch
+// per pass and axis length (k_*pass with a MultiTable).  A launch's blocks are the
 // concatenation of every member volume's blocks, and each block finds its volume in a
-// device-side table.  The whole n_iter sequence is captured once into a graph and
-// replayed on later calls with the same arguments.
+// device-side table.  The whole n_iter sequence is captured once into a graph and replayed on
+// later calls with the same arguments.
 
 namespace {
 
@@ -2512,11 +2787,17 @@ struct ZGroup {
     int shape;
 };
 
-// One all-lengths launch: the volumes of one length class
-template <class Args>
-struct LensGroup {
-    int cls;
-    LensTable<Args> *tab;
+// One launch of the fused form: the planes of the volumes of one size group, or the p-axis
+// convolutions of all volumes
+struct PlaneGroup {
+    int threads;
+    size_t smem;
+    PlaneTable *tab;
+    int64_t blocks;
+};
+struct ConvGroup {
+    size_t smem;
+    ConvTable *tab;
     int64_t blocks;
 };
 
@@ -2529,9 +2810,8 @@ struct BatchState {
     std::vector<XGroup> gx;
     std::vector<YGroup> gy;
     std::vector<ZGroup> gz;
-    std::vector<LensGroup<XArgs>> lx;
-    std::vector<LensGroup<YArgs>> ly;
-    std::vector<LensGroup<ZArgs>> lz;
+    std::vector<PlaneGroup> fp;
+    std::vector<ConvGroup> fc;
     void *dmem = nullptr;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
@@ -2558,18 +2838,18 @@ static cubic_status_t enqueue_batched(BatchState &b, cudaStream_t st)
     }
     if (b.n_iter == 0) return CUBIC_OK;
     auto xstage = [&](int mode) -> cubic_status_t {
-        for (const auto &g : b.lx) CUBIC_CUDA(launch_x_lens(g.cls, mode, g.tab, g.blocks, st));
+        for (const PlaneGroup &g : b.fp)
+            CUBIC_CUDA(launch_plane(mode, PlaneArgs{}, g.tab, g.blocks, g.threads, g.smem, st));
         for (const XGroup &g : b.gx) CUBIC_CUDA(g.k->xv[g.shape].m[mode](g.tab, g.blocks, st));
         return CUBIC_OK;
     };
     auto ystage = [&](int inverse) -> cubic_status_t {
-        for (const auto &g : b.ly) CUBIC_CUDA(launch_y_lens(g.cls, g.tab, g.blocks, inverse, st));
         for (const YGroup &g : b.gy) CUBIC_CUDA(g.k->yzv[g.shape].ym(g.tab, g.blocks, inverse, st));
         return CUBIC_OK;
     };
     auto yzy = [&](int zmode) -> cubic_status_t {
+        for (const ConvGroup &g : b.fc) CUBIC_CUDA(launch_conv(ConvArgs{}, g.tab, g.blocks, zmode, g.smem, st));
         if (cubic_status_t e = ystage(0)) return e;
-        for (const auto &g : b.lz) CUBIC_CUDA(launch_z_lens(g.cls, g.tab, g.blocks, zmode, st));
         for (const ZGroup &g : b.gz) CUBIC_CUDA(g.k->yzv[g.shape].zm(g.tab, g.blocks, zmode, st));
         return ystage(1);
     };
@@ -2674,9 +2954,8 @@ static int64_t fill_ztable(const BatchState &b, const std::vector<int> &vols, co
 
 using LenGroups = std::map<int64_t, std::vector<int>>;
 
-// Host tables of the all-lengths launches of one class (volumes in order of length);
-// each returns the launch's block count.
-static int64_t fill_lens_x(const BatchState &b, const std::vector<int> &vols, LensTable<XArgs> *t)
+// Host tables of the fused launches; each returns the launch's block count.
+static int64_t fill_plane(const BatchState &b, const std::vector<int> &vols, PlaneTable *t)
 {
     t->nvol = (int)vols.size();
     int64_t blocks = 0;
@@ -2690,44 +2969,33 @@ static int64_t fill_lens_x(const BatchState &b, const std::vector<int> &vols, Le
         a.dst = b.outs[vols[i]];
         a.d = b.images[vols[i]];
         a.eps = b.eps;
-        t->args[i] = a;
-        t->len[i] = (int)p->nx;
+        center_ratio(p, a);
+        t->args[i] = plane_args(p, a);
         t->prefix[i] = blocks;
-        blocks += lens_x_blocks((int)p->nx, p->rows);
+        blocks += p->fuse.g.np;
     }
     t->prefix[t->nvol] = blocks;
     return blocks;
 }
 
-static int64_t fill_lens_y(const BatchState &b, const std::vector<int> &vols, LensTable<YArgs> *t)
+static int64_t fill_conv(const BatchState &b, const std::vector<int> &vols, ConvTable *t)
 {
     t->nvol = (int)vols.size();
     int64_t blocks = 0;
     for (int i = 0; i < t->nvol; ++i) {
         cubic_rl_plan_s *p = b.plans[vols[i]];
-        t->args[i] = y_args(p, p->ws, 0, 0, p->xh);
-        t->len[i] = (int)p->ny;
+        t->args[i] = conv_args(p, p->ws);
         t->prefix[i] = blocks;
-        blocks += lens_col_blocks((int)p->ny, p->nz * p->xh);
+        blocks += p->fuse.conv_blocks;
     }
     t->prefix[t->nvol] = blocks;
     return blocks;
 }
 
-static int64_t fill_lens_z(const BatchState &b, const std::vector<int> &vols, LensTable<ZArgs> *t)
-{
-    t->nvol = (int)vols.size();
-    int64_t blocks = 0;
-    for (int i = 0; i < t->nvol; ++i) {
-        cubic_rl_plan_s *p = b.plans[vols[i]];
-        t->args[i] = z_args(p, p->ws, ZM_CONV, 1.f, 0, p->xh);
-        t->len[i] = (int)p->nz;
-        t->prefix[i] = blocks;
-        blocks += lens_col_blocks((int)p->nz, p->ny * p->xh);
-    }
-    t->prefix[t->nvol] = blocks;
-    return blocks;
-}
+// Planes launch in groups by size, up to kGroupSmem: a launch has one shared-memory size, its
+// largest plane's, which sets how many CTAs share an SM (four, two, one).
+constexpr int kPlaneGroups = 3;
+constexpr int kGroupSmem[kPlaneGroups] = {55 * 1024, 112 * 1024, (int)kPlaneSmemMax};
 
 // Times every candidate shape of every group whose length has no chosen shape yet, on
 // the batch's own buffers, and records the fastest: X by a ratio and an update launch, Y
@@ -2825,38 +3093,61 @@ static cubic_status_t batch_tune(BatchState &b, const LenGroups &byx, const LenG
 static cubic_status_t build_batch(BatchState &b, cudaStream_t st)
 {
     const int n = (int)b.plans.size();
-    // all-lengths classes where the axis length has one (their line indices are 32-bit),
-    // else a launch per length
+    // the fused form where it serves the volume, else a launch per pass and length
     LenGroups byx, byy, byz;
-    LenGroups lensx[kLensClasses], lensy[kLensClasses], lensz[kLensClasses];  // class -> length -> volumes
-    const int64_t kLines32 = (int64_t)1 << 31;
+    std::vector<int> planes[kPlaneGroups], convs;  // the fused form's launches
     for (int v = 0; v < n; ++v) {
         const cubic_rl_plan_s *p = b.plans[v];
-        const int cx = lens_class(p->nx), cy = lens_class(p->ny), cz = lens_class(p->nz);
-        if (cx >= 0) lensx[cx][p->nx].push_back(v);
-        else byx[p->nx].push_back(v);
-        if (cy >= 0 && p->nz * p->xh < kLines32) lensy[cy][p->ny].push_back(v);
-        else byy[p->ny].push_back(v);
-        if (cz >= 0 && p->ny * p->xh < kLines32) lensz[cz][p->nz].push_back(v);
-        else byz[p->nz].push_back(v);
+        if (p->fuse.ok) {
+            int i = 0;
+            while (p->fuse.g.smem > kGroupSmem[i]) ++i;
+            planes[i].push_back(v);
+            convs.push_back(v);
+            continue;
+        }
+        byx[p->nx].push_back(v);
+        byy[p->ny].push_back(v);
+        byz[p->nz].push_back(v);
     }
     cubic_status_t s = batch_tune(b, byx, byy, byz, st);
     if (s != CUBIC_OK) return s;
-    auto flat = [](const LenGroups &g) {
-        std::vector<int> vols;
-        for (auto &kv : g) vols.insert(vols.end(), kv.second.begin(), kv.second.end());
-        return vols;
-    };
-    size_t nlens = 0;
-    for (int c = 0; c < kLensClasses; ++c) nlens += !lensx[c].empty() + !lensy[c].empty() + !lensz[c].empty();
-    const size_t ntab = byx.size() + byy.size() + byz.size() + nlens;
-    const size_t tsz = std::max({sizeof(MultiTable<XArgs>), sizeof(MultiTable<YArgs>), sizeof(MultiTable<ZArgs>),
-                                 sizeof(LensTable<XArgs>), sizeof(LensTable<YArgs>), sizeof(LensTable<ZArgs>)});
+    size_t nfused = 0;
+    for (const auto &g : planes) nfused += !g.empty();
+    nfused += !convs.empty();
+    const size_t ntab = byx.size() + byy.size() + byz.size() + nfused;
+    const size_t tsz = std::max({sizeof(PlaneTable), sizeof(ConvTable),
+                                 sizeof(MultiTable<XArgs>), sizeof(MultiTable<YArgs>), sizeof(MultiTable<ZArgs>)});
     const size_t stride = (tsz + 255) / 256 * 256;
     std::vector<unsigned char> host(stride * ntab, 0);
     CUBIC_CUDA(cudaMalloc(&b.dmem, host.size()));
     unsigned char *dbase = (unsigned char *)b.dmem;
     size_t slot = 0;
+    for (std::vector<int> &g : planes) {
+        if (g.empty()) continue;
+        // the largest planes first; volumes of equal lengths side by side take the same branches
+        auto key = [&](int v) {
+            const PlaneGeo &q = b.plans[v]->fuse.g;
+            return std::make_tuple(-q.smem, q.nx, q.nc);
+        };
+        std::sort(g.begin(), g.end(), [&](int v, int w) { return key(v) < key(w); });
+        PlaneGroup pg;
+        pg.smem = (size_t)b.plans[g[0]]->fuse.g.smem;
+        pg.threads = plane_cta_threads(pg.smem, 4);
+        pg.tab = reinterpret_cast<PlaneTable *>(dbase + slot * stride);
+        pg.blocks = fill_plane(b, g, reinterpret_cast<PlaneTable *>(host.data() + slot * stride));
+        b.fp.push_back(pg);
+        ++slot;
+    }
+    if (!convs.empty()) {
+        std::sort(convs.begin(), convs.end(), [&](int v, int w) { return b.plans[v]->fuse.g.np > b.plans[w]->fuse.g.np; });
+        ConvGroup cg;
+        cg.smem = 0;
+        for (int v : convs) cg.smem = std::max(cg.smem, b.plans[v]->fuse.conv_smem);
+        cg.tab = reinterpret_cast<ConvTable *>(dbase + slot * stride);
+        cg.blocks = fill_conv(b, convs, reinterpret_cast<ConvTable *>(host.data() + slot * stride));
+        b.fc.push_back(cg);
+        ++slot;
+    }
     for (auto &kv : byx) {
         const AxisKernels *k = find_axis(kv.first);
         const int shape = chosen_shape(kv.first, 0, default_xshape(k));
@@ -2881,30 +3172,9 @@ static cubic_status_t build_batch(BatchState &b, cudaStream_t st)
         b.gz.push_back({k, reinterpret_cast<MultiTable<ZArgs> *>(dbase + slot * stride), blocks, shape});
         ++slot;
     }
-    for (int c = 0; c < kLensClasses; ++c) {
-        if (!lensx[c].empty()) {
-            const int64_t blocks =
-                fill_lens_x(b, flat(lensx[c]), reinterpret_cast<LensTable<XArgs> *>(host.data() + slot * stride));
-            b.lx.push_back({c, reinterpret_cast<LensTable<XArgs> *>(dbase + slot * stride), blocks});
-            ++slot;
-        }
-        if (!lensy[c].empty()) {
-            const int64_t blocks =
-                fill_lens_y(b, flat(lensy[c]), reinterpret_cast<LensTable<YArgs> *>(host.data() + slot * stride));
-            b.ly.push_back({c, reinterpret_cast<LensTable<YArgs> *>(dbase + slot * stride), blocks});
-            ++slot;
-        }
-        if (!lensz[c].empty()) {
-            const int64_t blocks =
-                fill_lens_z(b, flat(lensz[c]), reinterpret_cast<LensTable<ZArgs> *>(host.data() + slot * stride));
-            b.lz.push_back({c, reinterpret_cast<LensTable<ZArgs> *>(dbase + slot * stride), blocks});
-            ++slot;
-        }
-    }
     auto too_many = [](int64_t blocks) { return blocks > 0x7fffffff; };
-    for (const auto &g : b.lx) if (too_many(g.blocks)) return fail(CUBIC_ERR_INVALID_ARG, "batch too large for one launch");
-    for (const auto &g : b.ly) if (too_many(g.blocks)) return fail(CUBIC_ERR_INVALID_ARG, "batch too large for one launch");
-    for (const auto &g : b.lz) if (too_many(g.blocks)) return fail(CUBIC_ERR_INVALID_ARG, "batch too large for one launch");
+    for (const auto &g : b.fp) if (too_many(g.blocks)) return fail(CUBIC_ERR_INVALID_ARG, "batch too large for one launch");
+    for (const auto &g : b.fc) if (too_many(g.blocks)) return fail(CUBIC_ERR_INVALID_ARG, "batch too large for one launch");
     CUBIC_CUDA(cudaMemcpy(b.dmem, host.data(), host.size(), cudaMemcpyHostToDevice));
     return CUBIC_OK;
 }
@@ -3086,6 +3356,16 @@ extern "C" cubic_status_t cubic_rl_deconvolve_noalloc(const int64_t dims[3], con
     p.tw_z = p.tw + p.nx + p.ny;
     p.partial = (double *)(base + err_bytes + 2 * spec_bytes + tw_bytes);
     tuned_variants(&p);
+    // the fused form where its constants fit in what the array has left; H is then kept in
+    // that layout alone
+    // (an armed test of the bounded waits takes the form that has them)
+    fuse_setup(&p);
+    if (g_skip_copy_ns.load(std::memory_order_relaxed)) p.fuse.ok = false;
+    if (need + align256(p.fuse.tab_elems * sizeof(float2)) > kNoAllocScratchBytes) p.fuse.ok = false;
+    if (p.fuse.ok) {
+        p.HF = p.H;
+        p.ftab = (float2 *)(base + need);
+    }
 
     // The array keeps the previous call's contents.  Everything but the error word is
     // rewritten below before it is read; the error word starts at zero (static
@@ -3095,6 +3375,7 @@ extern "C" cubic_status_t cubic_rl_deconvolve_noalloc(const int64_t dims[3], con
     k_twiddles<<<grid_for(p.ny, 128, 1 << 20), 128, 0, st>>>(p.tw_y, (int)p.ny);
     k_twiddles<<<grid_for(p.nz, 128, 1 << 20), 128, 0, st>>>(p.tw_z, (int)p.nz);
     CUBIC_CUDA(cudaGetLastError());
+    if (p.fuse.ok) CUBIC_CUDA(launch_plane_tables(&p, st));
     s = load_psf(&p, psf, st);
     if (s != CUBIC_OK) return s;
     return enqueue_rl(&p, image, n_iter, eps, out, p.ws, st);

@@ -225,67 +225,98 @@ __device__ __forceinline__ float2 mul_w(float2 x)
 
 // ------------------------------------------------------------ register DFTs
 // Forward DFT X[k] = sum_n x[n] W_R^{kn}, in place on v[0..R).
+//
+// PK: complex additions as one packed instruction (two float32 lanes; the same roundings).
+// Additions of a rotated operand stay scalar: there the rotation is free, a packed one would
+// pay two register moves.  The packed form is for kernels bound by instruction fetch and
+// issue on one butterfly per thread (the fused form); the kernels that hold a whole line's
+// elements per thread measured up to 2% slower with it at lengths 2160 and 2560.
 
-template <int R>
+template <bool PK>
+__device__ __forceinline__ float2 padd(float2 a, float2 b)
+{
+    if constexpr (PK) return __fadd2_rn(a, b);
+    return cadd(a, b);
+}
+template <bool PK>
+__device__ __forceinline__ float2 psub(float2 a, float2 b)
+{
+    if constexpr (PK) return __ffma2_rn(b, make_float2(-1.f, -1.f), a);
+    return csub(a, b);
+}
+template <bool PK>
+__device__ __forceinline__ float2 pfma(float c, float2 a, float2 b)  // c a + b
+{
+    if constexpr (PK) return __ffma2_rn(make_float2(c, c), a, b);
+    return make_float2(fmaf(c, a.x, b.x), fmaf(c, a.y, b.y));
+}
+
+template <int R, bool PK = false>
 struct Dft;
 
-template <>
-struct Dft<1> {
+template <bool PK>
+struct Dft<1, PK> {
     __device__ __forceinline__ static void run(float2 (&)[1]) {}
 };
 
-template <>
-struct Dft<2> {
+template <bool PK>
+struct Dft<2, PK> {
     __device__ __forceinline__ static void run(float2 (&v)[2])
     {
         float2 a = v[0], b = v[1];
-        v[0] = cadd(a, b);
-        v[1] = csub(a, b);
+        v[0] = padd<PK>(a, b);
+        v[1] = psub<PK>(a, b);
     }
 };
 
-template <>
-struct Dft<3> {
+template <bool PK>
+struct Dft<3, PK> {
     __device__ __forceinline__ static void run(float2 (&v)[3])
     {
         constexpr float s3 = float(0.86602540378443864676);  // sin(2 pi / 3)
-        float2 a = v[0], t1 = cadd(v[1], v[2]), t2 = csub(v[1], v[2]);
-        float2 m = make_float2(fmaf(-0.5f, t1.x, a.x), fmaf(-0.5f, t1.y, a.y));
+        float2 a = v[0], t1 = padd<PK>(v[1], v[2]), t2 = psub<PK>(v[1], v[2]);
+        float2 m = pfma<PK>(-0.5f, t1, a);
         float2 j = make_float2(s3 * t2.y, -s3 * t2.x);  // -i sin(2pi/3) (x1 - x2)
-        v[0] = cadd(a, t1);
+        v[0] = padd<PK>(a, t1);
         v[1] = cadd(m, j);
         v[2] = csub(m, j);
     }
 };
 
-template <>
-struct Dft<4> {
+template <bool PK>
+struct Dft<4, PK> {
     __device__ __forceinline__ static void run(float2 (&v)[4])
     {
-        float2 s02 = cadd(v[0], v[2]), d02 = csub(v[0], v[2]);
-        float2 s13 = cadd(v[1], v[3]), d13 = mul_mi(csub(v[1], v[3]));
-        v[0] = cadd(s02, s13);
-        v[2] = csub(s02, s13);
+        float2 s02 = padd<PK>(v[0], v[2]), d02 = psub<PK>(v[0], v[2]);
+        float2 s13 = padd<PK>(v[1], v[3]), d13 = mul_mi(psub<PK>(v[1], v[3]));
+        v[0] = padd<PK>(s02, s13);
+        v[2] = psub<PK>(s02, s13);
         v[1] = cadd(d02, d13);
         v[3] = csub(d02, d13);
     }
 };
 
-template <>
-struct Dft<5> {
+template <bool PK>
+struct Dft<5, PK> {
     __device__ __forceinline__ static void run(float2 (&v)[5])
     {
         constexpr CtCis w1 = ct_cis(1, 5), w2 = ct_cis(2, 5);
         constexpr float c1 = float(w1.c), s1 = float(w1.s), c2 = float(w2.c), s2 = float(w2.s);
         float2 a = v[0];
-        float2 p1 = cadd(v[1], v[4]), m1 = csub(v[1], v[4]);
-        float2 p2 = cadd(v[2], v[3]), m2 = csub(v[2], v[3]);
-        float2 r1 = make_float2(a.x + c1 * p1.x + c2 * p2.x, a.y + c1 * p1.y + c2 * p2.y);
-        float2 r2 = make_float2(a.x + c2 * p1.x + c1 * p2.x, a.y + c2 * p1.y + c1 * p2.y);
+        float2 p1 = padd<PK>(v[1], v[4]), m1 = psub<PK>(v[1], v[4]);
+        float2 p2 = padd<PK>(v[2], v[3]), m2 = psub<PK>(v[2], v[3]);
+        float2 r1, r2;
+        if constexpr (PK) {
+            r1 = pfma<PK>(c2, p2, pfma<PK>(c1, p1, a));
+            r2 = pfma<PK>(c1, p2, pfma<PK>(c2, p1, a));
+        } else {
+            r1 = make_float2(a.x + c1 * p1.x + c2 * p2.x, a.y + c1 * p1.y + c2 * p2.y);
+            r2 = make_float2(a.x + c2 * p1.x + c1 * p2.x, a.y + c2 * p1.y + c1 * p2.y);
+        }
         // -i (s1 m1 + s2 m2) and -i (s2 m1 - s1 m2)
         float2 i1 = make_float2(s1 * m1.y + s2 * m2.y, -(s1 * m1.x + s2 * m2.x));
         float2 i2 = make_float2(s2 * m1.y - s1 * m2.y, -(s2 * m1.x - s1 * m2.x));
-        v[0] = cadd(a, cadd(p1, p2));
+        v[0] = padd<PK>(a, padd<PK>(p1, p2));
         v[1] = cadd(r1, i1);
         v[4] = csub(r1, i1);
         v[2] = cadd(r2, i2);
@@ -295,7 +326,7 @@ struct Dft<5> {
 
 // Composite R = A*B: A-point DFTs over n1 for every n2 (input n = n2 + B*n1),
 // twiddle W_R^{n2 k1}, then B-point DFTs over n2; output k = k1 + A*k2.
-template <int R>
+template <int R, bool PK>
 struct Dft {
     static constexpr int A = smallest_radix(R);
     static constexpr int B = R / A;
@@ -310,7 +341,7 @@ struct Dft {
                 constexpr int n1 = CUBIC_CI(n1_);
                 s[n1] = v[n2 + B * n1];
             });
-            Dft<A>::run(s);
+            Dft<A, PK>::run(s);
             static_for<0, A>([&](auto k1_) {
                 constexpr int k1 = CUBIC_CI(k1_);
                 y[n2][k1] = mul_w<n2 * k1, R>(s[k1]);
@@ -323,7 +354,7 @@ struct Dft {
                 constexpr int n2 = CUBIC_CI(n2_);
                 t[n2] = y[n2][k1];
             });
-            Dft<B>::run(t);
+            Dft<B, PK>::run(t);
             static_for<0, B>([&](auto k2_) {
                 constexpr int k2 = CUBIC_CI(k2_);
                 v[k1 + A * k2] = t[k2];

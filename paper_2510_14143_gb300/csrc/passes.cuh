@@ -86,6 +86,12 @@ struct XArgs {
     // transform (t = 0)
     const float *adj_u, *adj_q, *adj_b;
     float *adj_w, *adj_dbar;
+    // the fused form's plain iterations (null: not used): H at frequency zero over h0_scale.
+    // The ratio pass then transforms r - 1 and the update pass adds the PSF's sum back to q,
+    // which is the same correlation; the ratio is close to 1, so what is transformed, and
+    // with it the transforms' rounding error, is several times smaller
+    const float2 *h0;
+    float h0_scale;
 };
 
 struct YArgs {
@@ -193,14 +199,12 @@ constexpr bool x_uses_tma()
 }
 
 // shared memory: [2 mbarriers | operand rows (TMA modes) | stage twiddles | line-pair regions]
-// T: threads of the CTA.  Where T > P * L the threads past the L line pairs share one
-// spare line-pair region (they transform garbage there and touch no global memory).
-template <int N, int P, int L, int MODE, bool PF = false, int T = P * L>
+template <int N, int P, int L, int MODE, bool PF = false>
 constexpr size_t x_smem_bytes()
 {
     return 16 + (x_uses_tma<N, MODE, PF>() ? (size_t)L * 2 * N * sizeof(float) : 0) +
            (size_t)((tw_table_size(N, N / P) + 1) / 2 * 2) * sizeof(float2) +
-           (size_t)(L + (T > P * L ? 1 : 0)) * x_smem_line<N, P>() * sizeof(float2);
+           (size_t)L * x_smem_line<N, P>() * sizeof(float2);
 }
 
 // Merges two compensated sums over the T threads of the CTA, in a fixed order
@@ -260,13 +264,10 @@ __device__ __forceinline__ void slot_add(float *pair, CFloat v)
     catomic_add(pair, pair + 1, -v.c);
 }
 
-// T: threads of the CTA, P * L or more (the extra threads idle through the transforms on
-// a spare line-pair region, so that every thread meets every barrier)
-template <int N, int P, int L, int MODE, bool PF, int T = P * L>
+template <int N, int P, int L, int MODE, bool PF>
 __device__ __forceinline__ void x_body(const XArgs &a, const int64_t block)
 {
-    static_assert(T >= P * L && T < P * (L + 1), "a CTA of T threads holds L line pairs");
-    constexpr int E = N / P;
+    constexpr int E = N / P, T = P * L;  // threads of the CTA
     constexpr bool kTma = x_uses_tma<N, MODE, PF>();
     constexpr bool kPf = x_prefetches<N, MODE, PF>();
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -282,8 +283,7 @@ __device__ __forceinline__ void x_body(const XArgs &a, const int64_t block)
     const int l = threadIdx.x / P;
     const int64_t m = block * L + l;
     const int64_t r0 = 2 * m, r1 = 2 * m + 1;
-    const bool live = T == P * L || l < L;
-    const bool ok0 = live && r0 < a.rows, ok1 = live && r1 < a.rows;
+    const bool ok0 = r0 < a.rows, ok1 = r1 < a.rows;
     // image row -> spectrum row (row indices stay below 2^32: nz, ny <= 65535)
     auto srow = [&](int64_t r) -> int64_t {
         if (a.ny_img <= 0) return r;
