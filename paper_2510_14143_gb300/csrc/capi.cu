@@ -812,6 +812,7 @@ static void tune_load_locked()
 
 static void tuned_variants(cubic_rl_plan_s *p)
 {
+    p->vx = p->kx->dx;
     std::lock_guard<std::mutex> lk(g_tune_mu);
     tune_load_locked();
     for (const TuneEntry &e : g_tune)
@@ -3040,6 +3041,7 @@ static cubic_status_t batch_tune(BatchState &b, const LenGroups &byx, const LenG
         int best = default_xshape(k);
         float best_ms = 1e30f;
         for (int v = 0; v < k->nx && s == CUBIC_OK; ++v) {
+            if (!k->xv[v].m[XM_RATIO]) continue;
             auto *t = reinterpret_cast<MultiTable<XArgs> *>(host.data());
             const int64_t blocks = fill_xtable(b, kv.second, k, v, t);
             if ((s = upload()) != CUBIC_OK) break;

@@ -16,6 +16,7 @@
 
 #include "colpass_tma.cuh"
 #include "passes.cuh"
+#include "xwarp.cuh"
 
 namespace cubic {
 
@@ -31,7 +32,7 @@ constexpr int kMaxVariants = 8;
 struct XVariant {
     int P = 0, L = 0;
     XLaunch fn[XM_COUNT] = {};
-    XMultiLaunch m[XM_COUNT] = {};  // the same kernels over a table of volumes
+    XMultiLaunch m[XM_COUNT] = {};  // the same kernels over a table of volumes (null: single volume only)
 };
 
 struct YZVariant {
@@ -48,6 +49,7 @@ struct YZVariant {
 struct AxisKernels {
     int n = 0;
     int nx = 0, nyz = 0;  // number of X and Y/Z variants
+    int dx = 0;           // the X variant of a plan that was not tuned
     XVariant xv[kMaxVariants];
     YZVariant yzv[kMaxVariants];
     // multi-volume launches (batched path): X with xv[0]'s shape, Y/Z with P0 x 16 columns
@@ -102,6 +104,17 @@ cudaError_t launch_x(const XArgs &a, cudaStream_t st)
     if (attr != cudaSuccess) return attr;
     if (grid == 0) return cudaSuccess;
     return launch_pdl(fn, dim3((unsigned)grid), dim3(P * L), smem, st, a, (const MultiTable<XArgs> *)nullptr);
+}
+
+template <int N, int MODE>
+cudaError_t launch_xwarp(const XArgs &a, cudaStream_t st)
+{
+    constexpr int64_t L = kXWarps * xwarp_lines<N>();
+    const int64_t grid = ((a.rows + 1) / 2 + L - 1) / L;
+    static cudaError_t attr = set_smem((const void *)k_xwarp<N, MODE>, xwarp_smem<N>());
+    if (attr != cudaSuccess) return attr;
+    if (grid == 0) return cudaSuccess;
+    return launch_pdl(k_xwarp<N, MODE>, dim3((unsigned)grid), dim3(kXWarps * 32), xwarp_smem<N>(), st, a);
 }
 
 template <int N, int P, int B>
@@ -383,6 +396,21 @@ XVariant make_xvariant()
     return v;
 }
 
+// the warp-per-line kernels (single volume)
+template <int N>
+XVariant make_xvariant_warp()
+{
+    XVariant v;
+    v.P = 32 / xwarp_lines<N>();
+    v.L = kXWarps * xwarp_lines<N>();
+    v.fn[XM_FWD] = launch_xwarp<N, XM_FWD>;
+    v.fn[XM_INV] = launch_xwarp<N, XM_INV>;
+    v.fn[XM_RATIO] = launch_xwarp<N, XM_RATIO>;
+    v.fn[XM_UPDATE] = launch_xwarp<N, XM_UPDATE>;
+    v.fn[XM_FINAL] = launch_xwarp<N, XM_FINAL>;
+    return v;
+}
+
 template <int N, int P, int B>
 YZVariant make_yzvariant()
 {
@@ -458,6 +486,12 @@ AxisKernels make_axis()
         // the split with more elements per thread (fewer stages, fewer instructions) is held
         // to few CTAs per SM by its staged operand rows: both prefetched
         if constexpr (S::kAlt && N <= 1024) push_x(k, make_xvariant<N, P0, S::lines(P0, 128), true, true>());
+    }
+    // The warp-per-line kernels, the default where they exist: at every one of these lengths
+    // they are as fast as the best of the shapes above, or faster
+    if constexpr (xwarp_has(N)) {
+        k.dx = k.nx;
+        push_x(k, make_xvariant_warp<N>());
     }
     constexpr int XL = S::lines(P0, 128);
     k.xm[XM_FWD] = launch_x_multi<N, P0, XL, XM_FWD>;

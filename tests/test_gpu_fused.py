@@ -1,4 +1,6 @@
-"""The fused form (one plane kernel and one convolution kernel per half iteration) against the
+"""The fused form and the warp-per-line X kernels.
+
+The fused form (one plane kernel and one convolution kernel per half iteration) against the
 FP64 oracle and against the pass-by-pass form, at the lengths where it can go wrong: both
 choices of the in-plane axis, odd x, odd in-plane axes, butterflies that leave lanes of a warp
 idle, the smallest and largest radices, lengths and planes.
@@ -124,3 +126,34 @@ def test_psf_update_changes_both_forms(cr):
             cr.cubic_rl_convolve(plan, x, True, out)
         assert rel_l2(a, b) <= 1e-5
         assert rel_l2(a, oracle.convolve(oracle.psf_spectrum(psf), x.cpu().numpy(), True)) <= 1e-5
+
+
+# ---- the warp-per-line X kernels: the last X shape of these lengths, odd row counts and a
+# linear plan's row mapping included
+@pytest.mark.parametrize("n", [256, 320, 384, 512, 640, 768, 1024])
+@pytest.mark.parametrize("zy", [(3, 5), (2, 8), (9, 25)])
+def test_warp_per_line_x(cr, n, zy):
+    shape = zy + (n,)
+    psf = skewed_psf(shape, n + sum(zy))
+    plan = cr.cubic_rl_plan(shape, dev(psf))
+    (nx, _, _), _ = cr.cubic_rl_plan_variants(plan)
+    cr.cubic_rl_plan_set_variants(plan, nx - 1, 0, 0)
+    x = synth.random_field(shape, n, -1.0, 2.0)
+    out, u = (torch.full(shape, float("nan"), device="cuda") for _ in range(2))
+    for flipped in (False, True):
+        cr.cubic_rl_convolve(plan, dev(x), flipped, out)
+        assert rel_l2(out, oracle.convolve(oracle.psf_spectrum(psf), x, flipped)) <= 1e-5
+    d = synth.random_field(shape, 7, 5.0, 50.0)
+    cr.cubic_rl_deconvolve(plan, dev(d), 5, 1e-6, u)
+    assert rel_l2(u, oracle.rl(d, psf, 5, 1e-6)) <= 1e-5
+
+
+@pytest.mark.parametrize("nx", [250, 600])
+def test_warp_per_line_x_linear(cr, nx):
+    shape, k = (5, 7, nx), (3, 4, 9)
+    psf = skewed_psf(k, nx)
+    plan = cr.cubic_rl_plan_linear(shape, dev(psf))
+    d = synth.random_field(shape, nx, 5.0, 50.0)
+    u = torch.empty(shape, device="cuda")
+    cr.cubic_rl_deconvolve(plan, dev(d), 4, 1e-6, u)
+    assert rel_l2(u, oracle.rl_same(d, psf, 4, 1e-6)) <= 1e-5
