@@ -15,6 +15,7 @@
 #include <map>
 #include <mutex>
 #include <new>
+#include <numeric>
 #include <tuple>
 #include <vector>
 
@@ -2433,26 +2434,37 @@ __global__ void __launch_bounds__(256) k_ref_moments(const float *__restrict__ y
     }
 }
 
-// One iteration's record, merged in a fixed order: rec = (delta, nll s, nll c,
+// One iteration's record, merged in a fixed order by one warp: rec = (delta, nll s, nll c,
 // sx s, sx c, sxx s, sxx c, sxy s, sxy c) (value = s - c); ref_part may be null.
-__global__ void k_metrics(const float *__restrict__ dslots, const float *__restrict__ nslots,
-                          const float *__restrict__ ref_part, int nblk, float *__restrict__ rec)
+__device__ __forceinline__ CFloat warp_merge(CFloat v)
 {
-    if (threadIdx.x != 0) return;
-    CFloat num{0.f, 0.f}, den{0.f, 0.f}, nll{0.f, 0.f};
-    for (int i = 0; i < 64; ++i) {
+    for (int o = 16; o > 0; o >>= 1)
+        v = cf_merge(v, CFloat{__shfl_down_sync(0xffffffffu, v.s, o), __shfl_down_sync(0xffffffffu, v.c, o)});
+    return v;
+}
+
+__global__ void __launch_bounds__(32) k_metrics(const float *__restrict__ dslots, const float *__restrict__ nslots,
+                                                const float *__restrict__ ref_part, int nblk, float *__restrict__ rec)
+{
+    const int lane = threadIdx.x;
+    CFloat num{0.f, 0.f}, den{0.f, 0.f}, nll{0.f, 0.f}, r[3] = {};
+    for (int i = lane; i < 64; i += 32) {
         num = cf_merge(num, CFloat{dslots[4 * i], -dslots[4 * i + 1]});
         den = cf_merge(den, CFloat{dslots[4 * i + 2], -dslots[4 * i + 3]});
         nll = cf_merge(nll, CFloat{nslots[2 * i], -nslots[2 * i + 1]});
     }
+    if (ref_part)
+        for (int b = lane; b < nblk; b += 32)
+            for (int j = 0; j < 3; ++j) r[j] = cf_merge(r[j], CFloat{ref_part[6 * b + 2 * j], ref_part[6 * b + 2 * j + 1]});
+    num = warp_merge(num);
+    den = warp_merge(den);
+    nll = warp_merge(nll);
+    for (int j = 0; j < 3; ++j) r[j] = warp_merge(r[j]);
+    if (lane != 0) return;
     const float n = num.s - num.c, d = den.s - den.c;
     rec[0] = d > 0.f ? sqrtf(n / d) : 0.f;
     rec[1] = nll.s;
     rec[2] = nll.c;
-    CFloat r[3] = {};
-    if (ref_part)
-        for (int b = 0; b < nblk; ++b)
-            for (int j = 0; j < 3; ++j) r[j] = cf_merge(r[j], CFloat{ref_part[6 * b + 2 * j], ref_part[6 * b + 2 * j + 1]});
     for (int j = 0; j < 3; ++j) {
         rec[3 + 2 * j] = r[j].s;
         rec[4 + 2 * j] = r[j].c;
@@ -2609,35 +2621,87 @@ extern "C" cubic_status_t cubic_rl_deconvolve_monitor(cubic_rl_plan_t plan, cons
 
 constexpr int kFscMaxShells = 1024;
 
-// Shell sums in compensated float32: per block in shared memory, then into the
-// global pairs (value = hi + lo) -- sums[0..3S) high words, sums[3S..6S) low words.
+// Shell sums in compensated float32: per thread over a run of kx, per block in shared memory,
+// then into the global pairs (value = hi + lo) -- sums[0..3S) high words, sums[3S..6S) low
+// words.  A thread takes kFscRun adjacent kx of one row: the shell only grows along them, so
+// one exact search serves the run and the shared-memory atomics are one set per shell crossed
+// instead of one per element, with the lanes of a warp in different shells.  Integers: with L
+// the dims' least common multiple, rho^2 = rn / L^2, rn = sum (k L / n)^2; Int is int64 where
+// 3 S^2 L^2 fits it.
+constexpr int kFscRun = 8;
+
+template <class Int>
 __global__ void __launch_bounds__(256) k_fsc_bins(const float2 *__restrict__ A, const float2 *__restrict__ B,
-                                                  int64_t nz, int64_t ny, int64_t nx, int64_t xh, int64_t xp,
-                                                  int S, float *__restrict__ sums)
+                                                  int nz, int ny, int nx, int xh, int64_t xp, int64_t L, int S,
+                                                  float *__restrict__ sums)
 {
     extern __shared__ float sh_fsc[];  // [2][3][S]: high words, then low words
     for (int i = threadIdx.x; i < 6 * S; i += blockDim.x) sh_fsc[i] = 0.f;
     __syncthreads();
     float *lo = sh_fsc + 3 * S;
-    const int64_t cA = ny * ny * nx * nx, cB = nz * nz * nx * nx, cC = nz * nz * ny * ny;
-    const __int128 den = (__int128)cA * nz * nz;
-    const __int128 S4 = (__int128)4 * S * S;
-    const int64_t n = nz * ny * xh;
+    const int64_t fz = L / nz, fy = L / ny, fx = L / nx;
+    const Int den = (Int)L * L, S4 = (Int)4 * S * S;
+    const float scale = 2.f * (float)S / (float)L;
+    const unsigned nruns = (unsigned)(xh + kFscRun - 1) / kFscRun;
+    const int64_t n = (int64_t)nz * ny * nruns;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t kx = i % xh, row = i / xh, y = row % ny, z = row / ny;
-        const int64_t kz = 2 * z > nz ? z - nz : z, ky = 2 * y > ny ? y - ny : y;
-        const int64_t rn = kz * kz * cA + ky * ky * cB + kx * kx * cC;
-        const __int128 t = S4 * rn;  // shell s iff s^2 den <= t < (s+1)^2 den
-        if (t >= den * S * S) continue;  // rho >= 1/2
-        int sh = (int)(2.f * (float)S * sqrtf((float)rn / (float)den));  // estimate, corrected below
-        if (sh > S - 1) sh = S - 1;
-        while (sh > 0 && (__int128)sh * sh * den > t) --sh;
-        while (sh + 1 < S && (__int128)(sh + 1) * (sh + 1) * den <= t) ++sh;
-        const float w = (kx == 0 || 2 * kx == nx) ? 1.f : 2.f;
-        const float2 a = A[row * xp + kx], b = B[row * xp + kx];
-        catomic_add(&sh_fsc[sh], &lo[sh], w * (a.x * b.x + a.y * b.y));
-        catomic_add(&sh_fsc[S + sh], &lo[S + sh], w * (a.x * a.x + a.y * a.y));
-        catomic_add(&sh_fsc[2 * S + sh], &lo[2 * S + sh], w * (b.x * b.x + b.y * b.y));
+        const int64_t row = i / nruns;
+        const int k0 = (int)(i - row * nruns) * kFscRun, z = (int)(row / ny), y = (int)(row - (int64_t)z * ny);
+        const int64_t kz = (2 * z > nz ? z - nz : z) * fz, ky = (2 * y > ny ? y - ny : y) * fy;
+        const int64_t rzy = kz * kz + ky * ky;
+        // rows are 128-byte aligned and padded to 16 columns: the run loads whole
+        float2 a[kFscRun], b[kFscRun];
+        const float4 *a4 = reinterpret_cast<const float4 *>(A + row * xp + k0);
+        const float4 *b4 = reinterpret_cast<const float4 *>(B + row * xp + k0);
+#pragma unroll
+        for (int j = 0; j < kFscRun / 2; ++j) {
+            const float4 u = __ldg(a4 + j), v = __ldg(b4 + j);
+            a[2 * j] = make_float2(u.x, u.y);
+            a[2 * j + 1] = make_float2(u.z, u.w);
+            b[2 * j] = make_float2(v.x, v.y);
+            b[2 * j + 1] = make_float2(v.z, v.w);
+        }
+        const int64_t r0 = rzy + (int64_t)k0 * fx * ((int64_t)k0 * fx);
+        const Int t0 = S4 * r0;  // shell s iff s^2 den <= t < (s+1)^2 den
+        int sh = (int)(scale * sqrtf((float)r0));  // estimate, corrected below
+        if (sh > S) sh = S;
+        while (sh > 0 && (Int)sh * sh * den > t0) --sh;
+        CFloat ab{0.f, 0.f}, aa{0.f, 0.f}, bb{0.f, 0.f};
+        auto flush = [&] {
+            if (sh < S) {
+                catomic_add(&sh_fsc[sh], &lo[sh], ab.s);
+                catomic_add(&sh_fsc[S + sh], &lo[S + sh], aa.s);
+                catomic_add(&sh_fsc[2 * S + sh], &lo[2 * S + sh], bb.s);
+                if (ab.c != 0.f) atomicAdd(&lo[sh], -ab.c);
+                if (aa.c != 0.f) atomicAdd(&lo[S + sh], -aa.c);
+                if (bb.c != 0.f) atomicAdd(&lo[2 * S + sh], -bb.c);
+            }
+            ab = aa = bb = CFloat{0.f, 0.f};
+        };
+        Int next = (Int)(sh + 1) * (sh + 1) * den;
+        bool any = false;
+#pragma unroll
+        for (int j = 0; j < kFscRun; ++j) {
+            const int kx = k0 + j;
+            if (kx >= xh) break;
+            const int64_t x = (int64_t)kx * fx;
+            const Int t = S4 * (rzy + x * x);
+            if (t >= next) {
+                if (any) flush();
+                any = false;
+                while (sh < S && t >= next) {
+                    ++sh;
+                    next = (Int)(sh + 1) * (sh + 1) * den;
+                }
+            }
+            if (sh >= S) break;  // rho >= 1/2, here and further along
+            const float w = (kx == 0 || 2 * kx == nx) ? 1.f : 2.f;
+            ab = cf_add(ab, w * (a[j].x * b[j].x + a[j].y * b[j].y));
+            aa = cf_add(aa, w * (a[j].x * a[j].x + a[j].y * a[j].y));
+            bb = cf_add(bb, w * (b[j].x * b[j].x + b[j].y * b[j].y));
+            any = true;
+        }
+        if (any) flush();
     }
     __syncthreads();
     for (int i = threadIdx.x; i < 3 * S; i += blockDim.x) {
@@ -2686,8 +2750,12 @@ static cubic_status_t enqueue_fsc(cubic_rl_plan_s *p, const float *a, const floa
     if ((s = enqueue_forward3(p, a, p->ws, 1.f, st)) != CUBIC_OK) return s;
     if ((s = enqueue_forward3(p, b, p->ws2, 1.f, st)) != CUBIC_OK) return s;
     CUBIC_CUDA(cudaMemsetAsync(p->fsc_sums, 0, 6 * (size_t)n_shells * sizeof(float), st));
-    k_fsc_bins<<<grid_for(p->rows * p->xh, 256, 152 * 8), 256, 6 * n_shells * sizeof(float), st>>>(
-        p->ws, p->ws2, p->nz, p->ny, p->nx, p->xh, p->xp, n_shells, p->fsc_sums);
+    int64_t L = p->nx;
+    for (int64_t d : {p->ny, p->nz}) L = L / std::gcd(L, d) * d;
+    const unsigned grid = grid_for(p->rows * ((p->xh + kFscRun - 1) / kFscRun), 256, 152 * 4);
+    auto bins = 3.0 * n_shells * n_shells * (double)L * (double)L < 9e18 ? k_fsc_bins<int64_t> : k_fsc_bins<__int128>;
+    bins<<<grid, 256, 6 * n_shells * sizeof(float), st>>>(p->ws, p->ws2, (int)p->nz, (int)p->ny, (int)p->nx, (int)p->xh,
+                                                          p->xp, L, n_shells, p->fsc_sums);
     k_fsc_final<<<(n_shells + 255) / 256, 256, 0, st>>>(p->fsc_sums, n_shells, fsc);
     CUBIC_CUDA(cudaGetLastError());
     return CUBIC_OK;

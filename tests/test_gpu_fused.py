@@ -157,3 +157,14 @@ def test_warp_per_line_x_linear(cr, nx):
     u = torch.empty(shape, device="cuda")
     cr.cubic_rl_deconvolve(plan, dev(d), 4, 1e-6, u)
     assert rel_l2(u, oracle.rl_same(d, psf, 4, 1e-6)) <= 1e-5
+
+
+def test_fsc_long_common_multiple(cr):
+    # dims whose least common multiple sends the shell arithmetic past 64 bits
+    shape, shells = (125, 81, 256), 1024
+    a = synth.random_field(shape, 1, 0.0, 2.0)
+    b = a + synth.random_field(shape, 2, -1.0, 1.0)
+    psf = np.zeros(shape, np.float32)
+    psf[tuple(n // 2 for n in shape)] = 1
+    got = cr.cubic_fsc(cr.cubic_rl_plan(shape, dev(psf)), dev(a), dev(b), shells)
+    assert np.allclose(got.cpu().numpy(), oracle.fsc(a, b, shells)[0], atol=1e-4)
