@@ -2633,12 +2633,13 @@ constexpr int kFscRun = 8;
 template <class Int>
 __global__ void __launch_bounds__(256) k_fsc_bins(const float2 *__restrict__ A, const float2 *__restrict__ B,
                                                   int nz, int ny, int nx, int xh, int64_t xp, int64_t L, int S,
-                                                  float *__restrict__ sums)
+                                                  int copies, float *__restrict__ sums)
 {
-    extern __shared__ float sh_fsc[];  // [2][3][S]: high words, then low words
-    for (int i = threadIdx.x; i < 6 * S; i += blockDim.x) sh_fsc[i] = 0.f;
+    // [copies][2][3][S]: high words, then low words; a warp adds into one of the copies
+    extern __shared__ float smem_fsc[];
+    for (int i = threadIdx.x; i < 6 * S * copies; i += blockDim.x) smem_fsc[i] = 0.f;
     __syncthreads();
-    float *lo = sh_fsc + 3 * S;
+    float *sh_fsc = smem_fsc + (int)(threadIdx.x >> 5) % copies * 6 * S, *lo = sh_fsc + 3 * S;
     const int64_t fz = L / nz, fy = L / ny, fx = L / nx;
     const Int den = (Int)L * L, S4 = (Int)4 * S * S;
     const float scale = 2.f * (float)S / (float)L;
@@ -2705,8 +2706,11 @@ __global__ void __launch_bounds__(256) k_fsc_bins(const float2 *__restrict__ A, 
     }
     __syncthreads();
     for (int i = threadIdx.x; i < 3 * S; i += blockDim.x) {
-        if (sh_fsc[i] != 0.f) catomic_add(&sums[i], &sums[3 * S + i], sh_fsc[i]);
-        if (lo[i] != 0.f) catomic_add(&sums[i], &sums[3 * S + i], lo[i]);
+        CFloat t{0.f, 0.f};
+        for (int c = 0; c < copies; ++c)
+            t = cf_merge(t, CFloat{smem_fsc[c * 6 * S + i], -smem_fsc[c * 6 * S + 3 * S + i]});
+        if (t.s != 0.f) catomic_add(&sums[i], &sums[3 * S + i], t.s);
+        if (t.c != 0.f) catomic_add(&sums[i], &sums[3 * S + i], -t.c);
     }
 }
 
@@ -2753,9 +2757,11 @@ static cubic_status_t enqueue_fsc(cubic_rl_plan_s *p, const float *a, const floa
     int64_t L = p->nx;
     for (int64_t d : {p->ny, p->nz}) L = L / std::gcd(L, d) * d;
     const unsigned grid = grid_for(p->rows * ((p->xh + kFscRun - 1) / kFscRun), 256, 152 * 4);
+    const int set = 6 * n_shells * (int)sizeof(float);
+    const int copies = std::max(1, std::min(8, 40 * 1024 / set));  // of the block's sums
     auto bins = 3.0 * n_shells * n_shells * (double)L * (double)L < 9e18 ? k_fsc_bins<int64_t> : k_fsc_bins<__int128>;
-    bins<<<grid, 256, 6 * n_shells * sizeof(float), st>>>(p->ws, p->ws2, (int)p->nz, (int)p->ny, (int)p->nx, (int)p->xh,
-                                                          p->xp, L, n_shells, p->fsc_sums);
+    bins<<<grid, 256, copies * set, st>>>(p->ws, p->ws2, (int)p->nz, (int)p->ny, (int)p->nx, (int)p->xh, p->xp, L, n_shells,
+                                          copies, p->fsc_sums);
     k_fsc_final<<<(n_shells + 255) / 256, 256, 0, st>>>(p->fsc_sums, n_shells, fsc);
     CUBIC_CUDA(cudaGetLastError());
     return CUBIC_OK;
