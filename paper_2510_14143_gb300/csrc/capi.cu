@@ -814,6 +814,7 @@ static void tune_load_locked()
 static void tuned_variants(cubic_rl_plan_s *p)
 {
     p->vx = p->kx->dx;
+    p->vz = p->kz->dz;
     std::lock_guard<std::mutex> lk(g_tune_mu);
     tune_load_locked();
     for (const TuneEntry &e : g_tune)

@@ -49,7 +49,7 @@ struct YZVariant {
 struct AxisKernels {
     int n = 0;
     int nx = 0, nyz = 0;  // number of X and Y/Z variants
-    int dx = 0;           // the X variant of a plan that was not tuned
+    int dx = 0, dz = 0;  // the X and Z variants of a plan that was not tuned
     XVariant xv[kMaxVariants];
     YZVariant yzv[kMaxVariants];
     // multi-volume launches (batched path): X with xv[0]'s shape, Y/Z with P0 x 16 columns
@@ -533,6 +533,13 @@ AxisKernels make_axis()
                 push_yz(k, make_yzvariant_tma<N, P1, BY, NY1, 32, 2>());
         }
     }
+    // The Z shape of a plan that was not tuned (measured over volumes of 3 to 60 million voxels,
+    // us per launch, first shape -> this one): the split with at most 16 elements where that takes
+    // two radix stages (64 13.0 -> 12.2, 72 27.2 -> 23.4, 81 18.2 -> 16.0, 100 35.0 -> 33.2, 128
+    // 41.6 -> 37.7, 144 48.1 -> 45.6; with three or four stages it loses up to 60%).
+    if constexpr (S::kTuned && (BY > 0 || BZ > 0) && N <= 160 && S::P1 > 0 && S::P1 != P0 && S::P1 * 16 <= 1024)
+        if constexpr (plan_stages(N, N / S::P1) == 2 && tma_stages<N, P0, COL_Y>() <= 2 && tma_stages<N, P0, COL_Z>() <= 2)
+            k.dz = 1;
     push_yz(k, make_yzvariant<N, P0, B0>());
     // the wide plain shape as a tuning choice too (the reverse sweep's product passes run
     // on the widest plain variant)
@@ -541,6 +548,8 @@ AxisKernels make_axis()
         // short lines have one or two threads each: a TMA variant whose Z tile is 64
         // columns wide gives the CTA enough threads (thin stacks, e.g. 30 slices)
         push_yz(k, make_yzvariant_tma<N, P0, BY, 2, 64, 2>());
+        // the default Z shape of lengths 16 to 40 (1.1 to 1.75 times as fast as the first)
+        if constexpr (N >= 16 && N <= 40) k.dz = k.nyz - 1;
     }
     if constexpr (S::kTuned) {
         if constexpr (B0 == 16) push_yz(k, make_yzvariant<N, P0, 8>());
