@@ -533,15 +533,17 @@ static cudaError_t run_y(cubic_rl_plan_s *p, const YArgs &a, cudaStream_t st)
 {
     const double bytes = 2.0 * 8.0 * (double)p->rows * (double)(a.col1 - a.col0);
     YArgs b = a;
-    const YZVariant &yv = p->ky->yzv[p->vy];
-    if (yv.tma && yv.B > 0 && g_skip_copy_ns.load(std::memory_order_relaxed)) {
-        const unsigned long long ns = g_skip_copy_ns.exchange(0);
+    const YZVariant *yv = &p->ky->yzv[p->vy];
+    if (g_skip_copy_ns.load(std::memory_order_relaxed)) {
+        // an armed setting is taken by a tile pipeline: the first shape, where the default has none
+        if (!p->pinned && !yv->tma && p->ky->yzv[0].tma) yv = &p->ky->yzv[0];
+        const unsigned long long ns = yv->tma && yv->B > 0 ? g_skip_copy_ns.exchange(0) : 0;
         if (ns) {
             b.wait_ns = ns;
             b.skip_first = 1;
         }
     }
-    return counted(p, a.inverse ? KK_Y_INV : KK_Y_FWD, st, [&] { return p->ky->yzv[p->vy].y(b, st); }, bytes);
+    return counted(p, a.inverse ? KK_Y_INV : KK_Y_FWD, st, [&] { return yv->y(b, st); }, bytes);
 }
 
 static cudaError_t run_z(cubic_rl_plan_s *p, const ZArgs &a, cudaStream_t st)
@@ -814,6 +816,9 @@ static void tune_load_locked()
 static void tuned_variants(cubic_rl_plan_s *p)
 {
     p->vx = p->kx->dx;
+    // a linear plan's tiles leave the zero rows out of their copies (61x487x501 with a 25x33x33
+    // PSF, 20 iterations: 7.08 ms with the tile pipeline, 7.27 with the two-stage Y kernel)
+    p->vy = p->linear ? 0 : p->ky->dy;
     p->vz = p->kz->dz;
     std::lock_guard<std::mutex> lk(g_tune_mu);
     tune_load_locked();

@@ -17,6 +17,7 @@
 #include "colpass_tma.cuh"
 #include "passes.cuh"
 #include "xwarp.cuh"
+#include "yline.cuh"
 
 namespace cubic {
 
@@ -27,7 +28,7 @@ using XMultiLaunch = cudaError_t (*)(const MultiTable<XArgs> *, int64_t blocks, 
 using YMultiLaunch = cudaError_t (*)(const MultiTable<YArgs> *, int64_t blocks, int inverse, cudaStream_t);
 using ZMultiLaunch = cudaError_t (*)(const MultiTable<ZArgs> *, int64_t blocks, int mode, cudaStream_t);
 
-constexpr int kMaxVariants = 8;
+constexpr int kMaxVariants = 10;
 
 struct XVariant {
     int P = 0, L = 0;
@@ -49,7 +50,7 @@ struct YZVariant {
 struct AxisKernels {
     int n = 0;
     int nx = 0, nyz = 0;  // number of X and Y/Z variants
-    int dx = 0, dz = 0;  // the X and Z variants of a plan that was not tuned
+    int dx = 0, dy = 0, dz = 0;  // the X, Y and Z variants of a plan that was not tuned
     XVariant xv[kMaxVariants];
     YZVariant yzv[kMaxVariants];
     // multi-volume launches (batched path): X with xv[0]'s shape, Y/Z with P0 x 16 columns
@@ -115,6 +116,17 @@ cudaError_t launch_xwarp(const XArgs &a, cudaStream_t st)
     if (attr != cudaSuccess) return attr;
     if (grid == 0) return cudaSuccess;
     return launch_pdl(k_xwarp<N, MODE>, dim3((unsigned)grid), dim3(kXWarps * 32), xwarp_smem<N>(), st, a);
+}
+
+template <int N>
+cudaError_t launch_yline(const YArgs &a, cudaStream_t st)
+{
+    constexpr int B = yline_cols(N);
+    const dim3 grid((unsigned)((a.col1 - a.col0 + B - 1) / B), (unsigned)a.nz);
+    static cudaError_t attr = set_smem((const void *)k_yline<N>, yline_smem<N>());
+    if (attr != cudaSuccess) return attr;
+    if (grid.x == 0 || grid.y == 0) return cudaSuccess;
+    return launch_pdl(k_yline<N>, grid, dim3(yline_threads<N>()), yline_smem<N>(), st, a);
 }
 
 template <int N, int P, int B>
@@ -424,6 +436,18 @@ YZVariant make_yzvariant()
     return v;
 }
 
+// the two-stage Y kernel (single volume), with a plain shape for Z
+template <int N, int P, int B>
+YZVariant make_yzvariant_yline()
+{
+    YZVariant v;
+    v.P = P;
+    v.B = B;
+    v.y = launch_yline<N>;
+    v.z = launch_z<N, P, B>;
+    return v;
+}
+
 // ------------------------------------------------------------------ shapes
 
 inline void push_yz(AxisKernels &k, const YZVariant &v)
@@ -558,6 +582,10 @@ AxisKernels make_axis()
             if constexpr (N < 256) push_x(k, make_xvariant<N, P1, S::lines(P1, 128)>());
             constexpr int B1 = plain_cols<N, P1>() < 8 ? plain_cols<N, P1>() : 8;
             push_yz(k, make_yzvariant<N, P1, B1>());
+        }
+        if constexpr (yline_has(N)) {
+            if constexpr (yline_default(N)) k.dy = k.nyz;
+            push_yz(k, make_yzvariant_yline<N, P0, B0>());
         }
     }
     return k;

@@ -1,4 +1,4 @@
-"""The fused form and the warp-per-line X kernels.
+"""The fused form, the warp-per-line X kernels and the two-stage Y kernels.
 
 The fused form (one plane kernel and one convolution kernel per half iteration) against the
 FP64 oracle and against the pass-by-pass form, at the lengths where it can go wrong: both
@@ -168,3 +168,41 @@ def test_fsc_long_common_multiple(cr):
     psf[tuple(n // 2 for n in shape)] = 1
     got = cr.cubic_fsc(cr.cubic_rl_plan(shape, dev(psf)), dev(a), dev(b), shells)
     assert np.allclose(got.cpu().numpy(), oracle.fsc(a, b, shells)[0], atol=1e-4)
+
+
+# ---- the two-stage Y kernels: the last shape of these lengths; spectrum columns that leave
+# part of a column tile empty, a linear plan's rows that are not loaded or stored, column chunks
+Y_LENGTHS = [125, 128, 135, 144, 150, 160, 192, 256, 320, 384, 512, 640, 768, 1024]
+
+
+@pytest.mark.parametrize("n", Y_LENGTHS)
+@pytest.mark.parametrize("zx", [(2, 6), (3, 45), (1, 64)])
+def test_two_stage_y(cr, n, zx):
+    shape = (zx[0], n, zx[1])
+    psf = skewed_psf(shape, n + sum(zx))
+    plan = cr.cubic_rl_plan(shape, dev(psf))
+    (_, ny, _), _ = cr.cubic_rl_plan_variants(plan)
+    cr.cubic_rl_plan_set_variants(plan, 0, ny - 1, 0)
+    x = synth.random_field(shape, n, -1.0, 2.0)
+    out, u = (torch.full(shape, float("nan"), device="cuda") for _ in range(2))
+    for columns in (0, 16):
+        cr.cubic_rl_plan_set_chunk(plan, columns)
+        for flipped in (False, True):
+            cr.cubic_rl_convolve(plan, dev(x), flipped, out)
+            assert rel_l2(out, oracle.convolve(oracle.psf_spectrum(psf), x, flipped)) <= 1e-5, (columns, flipped)
+    d = synth.random_field(shape, 7, 5.0, 50.0)
+    cr.cubic_rl_deconvolve(plan, dev(d), 5, 1e-6, u)
+    assert rel_l2(u, oracle.rl(d, psf, 5, 1e-6)) <= 1e-5
+
+
+@pytest.mark.parametrize("ny", [121, 140, 187, 250, 301, 500, 1000])
+def test_two_stage_y_linear(cr, ny):
+    shape, k = (3, ny, 20), (3, 9, 5)
+    psf = skewed_psf(k, ny)
+    plan = cr.cubic_rl_plan_linear(shape, dev(psf))
+    (_, n, _), chosen = cr.cubic_rl_plan_variants(plan)
+    cr.cubic_rl_plan_set_variants(plan, chosen[0], n - 1, chosen[2])
+    d = synth.random_field(shape, ny, 5.0, 50.0)
+    u = torch.empty(shape, device="cuda")
+    cr.cubic_rl_deconvolve(plan, dev(d), 4, 1e-6, u)
+    assert rel_l2(u, oracle.rl_same(d, psf, 4, 1e-6)) <= 1e-5
