@@ -708,7 +708,7 @@ def load_traffic(kinds, w: synth.Workload):
 def source_hash() -> str:
     """Hash of the files the plain path's pass kernels compile from: the shard units and the
     headers they include (capi.cu, the host side and the small reduction kernels, and the
-    batched path's all-lengths kernels are left out)."""
+    fused form's kernels are left out)."""
     import glob
     import hashlib
     from paper_2510_14143_gb300 import build as _build

@@ -111,10 +111,10 @@ CUBIC_API cubic_status_t cubic_rl_deconvolve(cubic_rl_plan_t plan, const float *
 
 /* Batched Richardson-Lucy: the same deconvolution as cubic_rl_deconvolve for n volumes of
  * possibly different sizes, each with its own plan (plans must be distinct: a plan's scratch
- * serves one volume).  images[v], outs[v]: device float32 volumes of plans[v]'s dims.  For
- * each pass, the volumes whose length along that pass is one of the 5-smooth lengths 48 to
- * 160 share one kernel launch per length class (three classes by elements per thread, with
- * launch shapes fixed per length); the volumes of any other length share one launch per
+ * serves one volume).  images[v], outs[v]: device float32 volumes of plans[v]'s dims.  Small
+ * and medium volumes (axes of at most 192, an (x, y) or (x, z) plane of at most 122 KB) take the
+ * fused form, one plane kernel and one convolution kernel per half iteration over all of them;
+ * the volumes of any other size share one launch per pass and
  * length, whose launch shape (threads per line, lines or columns per CTA) is tuned the first
  * time the length appears: every candidate is timed on the call's own buffers and the
  * fastest is kept for the process.  A launch's blocks span every member volume.  The whole

@@ -13,7 +13,7 @@
 // 30.3; 192 17 -> 16.4 / 37.2 -> 33.8; 256 20.4 -> 17.0 / 47.4 -> 42.2; 320 24.5 -> 20.4 / 68.5 -> 66.6;
 // 384 26.4 -> 24.0 / 76.5 -> 81.6; 512 30.5 -> 28.6 / 104 -> 104; 640 45.0 -> 33.0 / 172 -> 145; 768 45.3
 // -> 39 / 178 -> 165; 1024 55.5 -> 50.2 / 190 -> 228.  256x256x128, a whole RL run of 100: 11.5 ->
-// 10.65 ms.  Lengths above 1024 (radices of 45 to 54, 6 warps per CTA, 4 columns) were up to 50%
+// 10.65 ms.  Lengths above 1024 (radices of 45 to 54, 6 warps per CTA, 4 columns) were 6 to 43%
 // slower than the tile pipeline and are not built.
 #pragma once
 
