@@ -53,7 +53,7 @@ def plans(cr, shape, psf):
     return fused, passes
 
 
-# (z, y, x): the plane takes the smaller of z and y (an odd one counts half as much again)
+# (z, y, x): the plane takes the smaller of z and y (an even one before an odd one)
 SHAPES = [(16, 20, 32), (20, 16, 36), (9, 24, 45), (10, 45, 75), (30, 25, 81), (81, 36, 135), (32, 27, 40), (8, 12, 50),
           (12, 8, 60), (24, 18, 125), (54, 100, 72), (40, 64, 72), (150, 160, 72), (144, 75, 64), (120, 160, 48),
           (45, 75, 64), (75, 81, 90), (81, 135, 75), (135, 75, 81), (45, 125, 80), (125, 45, 135), (12, 192, 192),
