@@ -120,7 +120,9 @@ CUBIC_API cubic_status_t cubic_rl_deconvolve(cubic_rl_plan_t plan, const float *
  * fastest is kept for the process.  A launch's blocks span every member volume.  The whole
  * n_iter sequence is captured once into a CUDA graph (first call with a given argument
  * set: tuning of new lengths, capture and instantiation, synchronous) and replayed on
- * `stream` by later calls with identical arguments (a few argument sets are cached).
+ * `stream` by later calls with identical arguments (a few argument sets are cached).  A plan
+ * that got another workspace or wait limit since, or whose PSF changed between symmetric and
+ * not, has its sequence captured anew; destroying a plan drops the graphs that run it.
  * 1 <= n <= 256.  Errors: INVALID_ARG, ALIGNMENT, OUT_OF_MEMORY, CUDA. */
 CUBIC_API cubic_status_t cubic_rl_deconvolve_batched(const cubic_rl_plan_t *plans, int n,
                                                      const float *const *images, int n_iter, float eps,

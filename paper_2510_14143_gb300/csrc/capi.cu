@@ -228,8 +228,15 @@ static const char *const kKindNames[KK_COUNT] = {
 
 // ------------------------------------------------------------------ plan
 
+// Numbers the states of all plans of the process: no two plans, and no two states of one plan
+// that a cached batch graph must tell apart, share one.
+static std::atomic<uint64_t> g_plan_state{1};
+
 struct cubic_rl_plan_s {
     int device = 0;
+    // renewed whenever something that the batched path's tables hold changes: work array, kind
+    // and buffers of H, wait limit
+    uint64_t state = g_plan_state.fetch_add(1);
     int64_t nz = 0, ny = 0, nx = 0, V = 0, rows = 0, xh = 0, xp = 0;
     const AxisKernels *kx = nullptr, *ky = nullptr, *kz = nullptr;
     int vx = 0, vy = 0, vz = 0; // launch-shape variant of each pass
@@ -730,7 +737,7 @@ static cubic_status_t load_fused_h(cubic_rl_plan_s *p, const float *h0, bool eve
     return CUBIC_OK;
 }
 
-static cubic_status_t load_psf(cubic_rl_plan_s *p, const float *psf, cudaStream_t st)
+static cubic_status_t rebuild_h(cubic_rl_plan_s *p, const float *psf, cudaStream_t st)
 {
     cubic_status_t s = ensure_workspace(p);
     if (s != CUBIC_OK) return s;
@@ -780,6 +787,16 @@ static cubic_status_t load_psf(cubic_rl_plan_s *p, const float *psf, cudaStream_
     CUBIC_CUDA(cudaGetLastError());
     p->use_real_h = true;
     return CUBIC_OK;
+}
+
+// Whether a batch graph multiplies by the real or the complex spectrum is fixed when it is
+// captured, so a change between the two is a new state of the plan.
+static cubic_status_t load_psf(cubic_rl_plan_s *p, const float *psf, cudaStream_t st)
+{
+    const bool real = p->use_real_h;
+    const cubic_status_t s = rebuild_h(p, psf, st);
+    if (p->use_real_h != real) p->state = g_plan_state.fetch_add(1);
+    return s;
 }
 
 // ------------------------------------------------------------------ tuning cache
@@ -995,10 +1012,13 @@ extern "C" cubic_status_t cubic_rl_plan_update_psf(cubic_rl_plan_t plan, const f
     return load_psf(plan, psf, (cudaStream_t)stream);
 }
 
+static void drop_batches(const cubic_rl_plan_s *p);
+
 extern "C" cubic_status_t cubic_rl_plan_destroy(cubic_rl_plan_t plan)
 {
     if (!plan) return CUBIC_OK;
     cudaDeviceSynchronize();
+    drop_batches(plan);
     cudaFree(plan->H);
     cudaFree(plan->tw);
     cudaFree(plan->partial);
@@ -1044,6 +1064,7 @@ extern "C" cubic_status_t cubic_rl_set_workspace(cubic_rl_plan_t plan, void *dev
     }
     plan->ws = (float2 *)dev_ptr;
     plan->own_ws = false;
+    plan->state = g_plan_state.fetch_add(1);
     return CUBIC_OK;
 }
 
@@ -1610,6 +1631,7 @@ extern "C" cubic_status_t cubic_rl_plan_set_wait_limit(cubic_rl_plan_t plan, uin
 {
     if (!plan) return fail(CUBIC_ERR_INVALID_ARG, "plan must be non-null");
     plan->wait_ns = limit_ns;
+    plan->state = g_plan_state.fetch_add(1);
     return CUBIC_OK;
 }
 
@@ -2884,6 +2906,7 @@ struct ConvGroup {
 
 struct BatchState {
     std::vector<cubic_rl_plan_s *> plans;
+    std::vector<uint64_t> states;  // of the plans when the tables were made
     std::vector<const float *> images;
     std::vector<float *> outs;
     int n_iter = 0;
@@ -2910,6 +2933,21 @@ std::vector<BatchState *> g_batches;  // most recent last; a few kept
 int64_t g_batch_last_nodes = 0;
 
 }  // namespace
+
+// Forgets the graphs that run plan p (the device is idle)
+static void drop_batches(const cubic_rl_plan_s *p)
+{
+    std::lock_guard<std::mutex> lk(g_batch_mu);
+    for (size_t i = 0; i < g_batches.size();) {
+        const auto &v = g_batches[i]->plans;
+        if (std::find(v.begin(), v.end(), p) == v.end()) {
+            ++i;
+            continue;
+        }
+        delete g_batches[i];
+        g_batches.erase(g_batches.begin() + (long)i);
+    }
+}
 
 static cubic_status_t enqueue_batched(BatchState &b, cudaStream_t st)
 {
@@ -3288,7 +3326,8 @@ extern "C" cubic_status_t cubic_rl_deconvolve_batched(const cubic_rl_plan_t *pla
         if ((int)b->plans.size() != n || b->n_iter != n_iter || b->eps != eps) continue;
         bool same = true;
         for (int v = 0; v < n && same; ++v)
-            same = b->plans[v] == plans[v] && b->images[v] == images[v] && b->outs[v] == outs[v];
+            same = b->plans[v] == plans[v] && b->states[v] == plans[v]->state && b->images[v] == images[v] &&
+                   b->outs[v] == outs[v];
         if (same) hit = b;
     }
     if (!hit) {
@@ -3299,6 +3338,7 @@ extern "C" cubic_status_t cubic_rl_deconvolve_batched(const cubic_rl_plan_t *pla
         BatchState *b = new (std::nothrow) BatchState();
         if (!b) return fail(CUBIC_ERR_OUT_OF_MEMORY, "host allocation failed");
         b->plans.assign(plans, plans + n);
+        for (int v = 0; v < n; ++v) b->states.push_back(plans[v]->state);
         b->images.assign(images, images + n);
         b->outs.assign(outs, outs + n);
         b->n_iter = n_iter;
