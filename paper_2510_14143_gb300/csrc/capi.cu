@@ -142,11 +142,15 @@ __global__ void k_center_to_origin(const float *__restrict__ psf, float *__restr
 constexpr int kReduceThreads = 256;
 constexpr int kReduceBlocks = 1024;
 
+// COUNT: also the number of values above zero, per block.
+template <bool COUNT>
 __global__ void __launch_bounds__(kReduceThreads) k_sum_partial(const float *__restrict__ x, int64_t n,
-                                                                double *__restrict__ partial)
+                                                                double *__restrict__ partial, unsigned *__restrict__ count)
 {
     __shared__ double sh[kReduceThreads / 32];
+    __shared__ unsigned sh_n[kReduceThreads / 32];
     CFloat a{0.f, 0.f}, b{0.f, 0.f};
+    unsigned above = 0;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t first = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     // 16-byte vectors where x is 16-byte aligned, then the scalar tail
@@ -156,32 +160,86 @@ __global__ void __launch_bounds__(kReduceThreads) k_sum_partial(const float *__r
         const float4 v = __ldg(x4 + i);
         a = cf_add(cf_add(a, v.x), v.y);
         b = cf_add(cf_add(b, v.z), v.w);
+        if (COUNT) above += (v.x > 0.f) + (v.y > 0.f) + (v.z > 0.f) + (v.w > 0.f);
     }
-    for (int64_t i = 4 * n4 + first; i < n; i += stride) a = cf_add(a, __ldg(x + i));
+    for (int64_t i = 4 * n4 + first; i < n; i += stride) {
+        const float v = __ldg(x + i);
+        a = cf_add(a, v);
+        if (COUNT) above += v > 0.f;
+    }
     double s = ((double)a.s - (double)a.c) + ((double)b.s - (double)b.c);
     for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
+    if (COUNT) above = __reduce_add_sync(0xffffffffu, above);
+    if ((threadIdx.x & 31) == 0) {
+        sh[threadIdx.x >> 5] = s;
+        sh_n[threadIdx.x >> 5] = above;
+    }
     __syncthreads();
     if (threadIdx.x < 32) {
         s = threadIdx.x < kReduceThreads / 32 ? sh[threadIdx.x] : 0.0;
         for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-        if (threadIdx.x == 0) partial[blockIdx.x] = s;
+        if (COUNT) above = __reduce_add_sync(0xffffffffu, threadIdx.x < kReduceThreads / 32 ? sh_n[threadIdx.x] : 0u);
+        if (threadIdx.x == 0) {
+            partial[blockIdx.x] = s;
+            if (COUNT) count[blockIdx.x] = above;
+        }
     }
 }
 
+// The constant that a plain iteration of the fused form takes off the ratio r = d / max(b, eps)
+// before its transform, and what that takes off the correlation (XArgs::center).  A transform's
+// rounding error is a fixed share of its input's size, and the ratio is nearly constant wherever
+// the image has light, so taking its mean off lowers the error.  At the start b = S u0 everywhere,
+// S the PSF's sum, and the mean of r is mean(d) / max(S u0, eps): 1 / S unless eps is at work.
+// Where d = 0, r = 0 from then on: the mean falls with the share of voxels that have light.  A
+// constant above twice the mean would raise the error (a constant of 1 with a PSF of sum 1000:
+// 4e-7 -> 6e-4 after 30 iterations of 32x64x64 voxels); none is taken off where S or the mean is
+// not a positive number.
+struct RatioCenter {
+    const float2 *h0 = nullptr;  // H at frequency zero, over h0_scale
+    float h0_scale = 0.f;
+    int64_t V = 0;
+    float eps = 0.f;
+    unsigned *count = nullptr;   // voxels above zero, per block of the sum
+    float2 *out = nullptr;       // the constant, and the constant times S
+};
+
+__device__ __forceinline__ float2 ratio_center(const RatioCenter &a, double sum, unsigned above)
+{
+    // any constant will do as long as both places use the same: float32 throughout
+    const float n = (float)a.V, mean = (float)sum / n, S = a.h0->x * a.h0_scale;
+    if (!(S > 0.f && mean > 0.f)) return make_float2(0.f, 0.f);
+    const float c = mean / fmaxf(S * fmaxf(mean, a.eps), a.eps) * ((float)above / n), h = c * S;
+    return c < INFINITY && h < INFINITY ? make_float2(c, h) : make_float2(0.f, 0.f);
+}
+
+template <bool COUNT>
 __global__ void __launch_bounds__(kReduceThreads) k_sum_final(const double *__restrict__ partial, int n,
-                                                              double *__restrict__ out)
+                                                              double *__restrict__ out, const RatioCenter center)
 {
     __shared__ double sh[kReduceThreads / 32];
+    __shared__ unsigned sh_n[kReduceThreads / 32];
     double s = 0.0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) s += partial[i];
+    unsigned above = 0;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        s += partial[i];
+        if (COUNT) above += center.count[i];
+    }
     for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
+    if (COUNT) above = __reduce_add_sync(0xffffffffu, above);
+    if ((threadIdx.x & 31) == 0) {
+        sh[threadIdx.x >> 5] = s;
+        sh_n[threadIdx.x >> 5] = above;
+    }
     __syncthreads();
     if (threadIdx.x < 32) {
         s = threadIdx.x < kReduceThreads / 32 ? sh[threadIdx.x] : 0.0;
         for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-        if (threadIdx.x == 0) out[0] = s;
+        if (COUNT) above = __reduce_add_sync(0xffffffffu, threadIdx.x < kReduceThreads / 32 ? sh_n[threadIdx.x] : 0u);
+        if (threadIdx.x == 0) {
+            out[0] = s;
+            if (COUNT) *center.out = ratio_center(center, s, above);
+        }
     }
 }
 
@@ -280,6 +338,7 @@ struct cubic_rl_plan_s {
         int64_t conv_blocks = 0;
         size_t conv_smem = 0;
         size_t tab_elems = 0;         // the constant block, float2
+        size_t off_center = 0;        // in it: the ratio's centre, then kReduceBlocks counts
         bool c_is_z = false;
     } fuse;
     float2 *ftab = nullptr;           // the fused form's constants (plane_tables), owned
@@ -422,7 +481,8 @@ static bool fuse_geometry(const cubic_rl_plan_s *p, bool c_is_z, cubic_rl_plan_s
     f->ok = true;
     f->g = g;
     f->c_is_z = c_is_z;
-    f->tab_elems = (size_t)g.off_plane + (size_t)v.tw;
+    f->off_center = (size_t)g.off_plane + (size_t)v.tw;
+    f->tab_elems = f->off_center + 1 + kReduceBlocks / 2;
     f->conv_blocks = conv_blocks_of(v, g.mv);
     f->conv_smem = conv_smem_of(ConvLens{}, np);
     // Warps per CTA: the fewest that run the fewest rounds of x and c tasks (weighted by a
@@ -605,13 +665,13 @@ static XArgs x_args(const cubic_rl_plan_s *p, bool full = false)
     return a;
 }
 
-// A plain iteration in the fused form takes 1 off the ratio before its transform and adds
-// the PSF's sum back to the correlation (XArgs::h0).  H carries 1 / 2V there.  Not in the
-// differentiable path, which needs the spectrum of the ratio itself.
+// A plain iteration in the fused form takes a constant off the ratio before its transform and
+// adds the constant times the PSF's sum back to the correlation (see RatioCenter; enqueue_init
+// has written both).  Not in the differentiable path, which needs the spectrum of the ratio
+// itself.
 static void center_ratio(const cubic_rl_plan_s *p, XArgs &a)
 {
-    a.h0 = p->HF;
-    a.h0_scale = (float)(2.0 * (double)p->V);
+    a.center = p->ftab + p->fuse.off_center;
 }
 
 // Forward 3D real-to-half-complex transform of `real` into `spec`, optionally
@@ -1081,12 +1141,26 @@ static bool ranges_overlap(const void *a, size_t na, const void *b, size_t nb)
     return x < y + nb && y < x + na;
 }
 
-// u0 = max(mean(image), eps) into out.
+// u0 = max(mean(image), eps) into out; where the fused form serves the plan, also the ratio's
+// centre (H carries 1 / 2V there).
 static cubic_status_t enqueue_init(cubic_rl_plan_s *p, const float *image, float eps, float *out, cudaStream_t st)
 {
     CUBIC_CUDA(counted(p, KK_SUM, st, [&] {
-        k_sum_partial<<<kReduceBlocks, kReduceThreads, 0, st>>>(image, p->V, p->partial);
-        k_sum_final<<<1, kReduceThreads, 0, st>>>(p->partial, kReduceBlocks, p->partial + kReduceBlocks);
+        double *sum = p->partial + kReduceBlocks;
+        if (p->fuse.ok) {
+            RatioCenter c;
+            c.h0 = p->HF;
+            c.h0_scale = (float)(2.0 * (double)p->V);
+            c.V = p->V;
+            c.eps = eps;
+            c.out = p->ftab + p->fuse.off_center;
+            c.count = reinterpret_cast<unsigned *>(c.out + 1);
+            k_sum_partial<true><<<kReduceBlocks, kReduceThreads, 0, st>>>(image, p->V, p->partial, c.count);
+            k_sum_final<true><<<1, kReduceThreads, 0, st>>>(p->partial, kReduceBlocks, sum, c);
+        } else {
+            k_sum_partial<false><<<kReduceBlocks, kReduceThreads, 0, st>>>(image, p->V, p->partial, nullptr);
+            k_sum_final<false><<<1, kReduceThreads, 0, st>>>(p->partial, kReduceBlocks, sum, RatioCenter());
+        }
         return cudaGetLastError();
     }));
     p->launches[KK_SUM] += 1;  // two kernels
@@ -1166,8 +1240,9 @@ static cubic_status_t lin_init(cubic_rl_plan_s *p, const float *image, float eps
     cubic_status_t s = lin_pad(p, image, dp, st);
     if (s != CUBIC_OK) return s;
     CUBIC_CUDA(counted(p, KK_SUM, st, [&] {
-        k_sum_partial<<<kReduceBlocks, kReduceThreads, 0, st>>>(dp, E, p->partial);
-        k_sum_final<<<1, kReduceThreads, 0, st>>>(p->partial, kReduceBlocks, p->partial + kReduceBlocks);
+        k_sum_partial<false><<<kReduceBlocks, kReduceThreads, 0, st>>>(dp, E, p->partial, nullptr);
+        k_sum_final<false><<<1, kReduceThreads, 0, st>>>(p->partial, kReduceBlocks, p->partial + kReduceBlocks,
+                                                         RatioCenter());
         return cudaGetLastError();
     }));
     CUBIC_CUDA(counted(p, KK_FILL, st, [&] {
@@ -1451,7 +1526,7 @@ extern "C" cubic_status_t cubic_psf_gaussian(const int64_t dims[3], float sigma_
     const float a_xy = (float)(0.5 / ((double)sigma_xy * sigma_xy));
     const float a_z = (float)(0.5 / ((double)sigma_z * sigma_z));
     k_psf_gauss<<<kReduceBlocks, kReduceThreads, 0, st>>>(psf, dims[0], dims[1], dims[2], a_xy, a_z, partial);
-    k_sum_final<<<1, kReduceThreads, 0, st>>>(partial, kReduceBlocks, partial + kReduceBlocks);
+    k_sum_final<false><<<1, kReduceThreads, 0, st>>>(partial, kReduceBlocks, partial + kReduceBlocks, RatioCenter());
     k_scale_by_sum<<<grid_for(V, 256), 256, 0, st>>>(psf, V, partial + kReduceBlocks, (double)amp);
     cudaError_t e = cudaGetLastError();
     cudaFreeAsync(scratch, st);
@@ -1975,8 +2050,8 @@ extern "C" cubic_status_t cubic_rl_backward(cubic_rl_plan_t plan, const float *i
         float *gsum = reinterpret_cast<float *>(gpart + kReduceBlocks);
         k_csum_partial<<<kReduceBlocks, kReduceThreads, 0, st>>>(g, V, gpart);
         k_csum_final<<<1, 32, 0, st>>>(gpart, kReduceBlocks, gsum);
-        k_sum_partial<<<kReduceBlocks, kReduceThreads, 0, st>>>(image, V, red);
-        k_sum_final<<<1, kReduceThreads, 0, st>>>(red, kReduceBlocks, red + kReduceBlocks);
+        k_sum_partial<false><<<kReduceBlocks, kReduceThreads, 0, st>>>(image, V, red, nullptr);
+        k_sum_final<false><<<1, kReduceThreads, 0, st>>>(red, kReduceBlocks, red + kReduceBlocks, RatioCenter());
         k_add_mean_grad<<<gr, 256, 0, st>>>(dbar, gsum, red + kReduceBlocks, V, eps);
         CUBIC_CUDA(cudaMemcpyAsync(grad_image, dbar, (size_t)V * sizeof(float), cudaMemcpyDeviceToDevice, st));
     }

@@ -176,10 +176,11 @@ __device__ __forceinline__ void plane_point(const XArgs &a, float2 (&v)[E], cons
             const float x1 = __fdividef(two ? __ldg(p1 + n) : 0.f, fmaxf(v[i].y, eps));
             v[i] = make_float2(x0, x1);
         });
-        if (a.h0) {
+        if (a.center) {
+            const float c = __ldg(&a.center->x);
             static_for<0, E>([&](auto i_) {
                 constexpr int i = CUBIC_CI(i_);
-                v[i] = make_float2(v[i].x - 1.f, two ? v[i].y - 1.f : 0.f);
+                v[i] = make_float2(v[i].x - c, two ? v[i].y - c : 0.f);
             });
         }
         if (a.keep_b) {
@@ -192,8 +193,8 @@ __device__ __forceinline__ void plane_point(const XArgs &a, float2 (&v)[E], cons
     } else if constexpr (MODE == XM_UPDATE || MODE == XM_FINAL) {
         float *ob = (MODE == XM_FINAL || a.dst) ? a.dst : a.u;
         const float *p0 = a.u + o0, *p1 = a.u + o1;
-        if (a.h0) {
-            const float h = __ldg(&a.h0->x) * a.h0_scale;
+        if (a.center) {
+            const float h = __ldg(&a.center->y);
             static_for<0, E>([&](auto i_) { v[CUBIC_CI(i_)] = cadd(v[CUBIC_CI(i_)], make_float2(h, h)); });
         }
         if (a.keep_a) {

@@ -86,12 +86,11 @@ struct XArgs {
     // transform (t = 0)
     const float *adj_u, *adj_q, *adj_b;
     float *adj_w, *adj_dbar;
-    // the fused form's plain iterations (null: not used): H at frequency zero over h0_scale.
-    // The ratio pass then transforms r - 1 and the update pass adds the PSF's sum back to q,
-    // which is the same correlation; the ratio is close to 1, so what is transformed, and
-    // with it the transforms' rounding error, is several times smaller
-    const float2 *h0;
-    float h0_scale;
+    // the fused form's plain iterations (null: not used): a constant x and y = x times the PSF's
+    // sum.  The ratio pass transforms r - x and the update pass adds y back to q, which is the
+    // same correlation; the ratio is mostly close to x, so what is transformed, and with it the
+    // transforms' rounding error, is smaller
+    const float2 *center;
 };
 
 struct YArgs {
