@@ -197,24 +197,35 @@ CUBIC_API cubic_status_t cubic_test_skip_next_tile_copy(uint64_t wait_ns);
 
 /* ---- launch shapes and autotuning ---- */
 
-/* counts[3] = number of compiled launch-shape variants of the X, Y and Z passes for this
- * plan's lengths; chosen[3] = the variants in use.  Either pointer may be NULL. */
+/* The launch shapes of the pass-by-pass form.  Small and medium circular volumes (axes of at
+ * most 192, an (x, y) or (x, z) plane of at most 122 KB) run in the fused form instead, which has
+ * no shapes to choose from: there the shapes serve cubic_rl_fft3_*, cubic_fsc and the PSF's
+ * transform, and plain calls only once cubic_rl_plan_set_variants has been called.
+ * counts[3] = number of compiled launch-shape variants of the X, Y and Z passes for this
+ * plan's lengths; chosen[3] = the chosen variants.  Either pointer may be NULL. */
 CUBIC_API cubic_status_t cubic_rl_plan_variants(cubic_rl_plan_t plan, int counts[3], int chosen[3]);
 
 /* Select launch-shape variants explicitly (INVALID_ARG if out of range).  Every variant
- * computes the same transform; they differ in threads per line and lines per CTA. */
+ * computes the same transform; they differ in threads per line and lines per CTA.  The plan
+ * runs its calls in the pass-by-pass form from then on, to the same float32 accuracy but not
+ * to the bit, whatever the variants; the batched call still takes the fused form where the
+ * volume's size allows it. */
 CUBIC_API cubic_status_t cubic_rl_plan_set_variants(cubic_rl_plan_t plan, int vx, int vy, int vz);
 
 /* Process the Y-forward / Z / Y-inverse passes of each convolution in chunks of `columns`
  * spectrum columns (a multiple of 16; 0 = all columns in one launch per pass), so that a
- * chunk stays in L2 between the three passes.  Results do not depend on it. */
+ * chunk stays in L2 between the three passes.  A chunk is rounded up to whole tiles of the
+ * launch shapes in use (at most 64 columns).  Chunks exist in the pass-by-pass form alone: a
+ * small or medium volume's plan leaves the fused form (see cubic_rl_plan_variants) while they
+ * are on.  Within that form results do not depend on them. */
 CUBIC_API cubic_status_t cubic_rl_plan_set_chunk(cubic_rl_plan_t plan, int64_t columns);
 
 /* Current chunk setting (-1 for a NULL plan). */
 CUBIC_API int64_t cubic_rl_plan_chunk(cubic_rl_plan_t plan);
 
 /* Time every variant of each pass on this plan's own buffers (image read, `out` and the
- * workspace overwritten) and keep the fastest.  Synchronises the stream several times, so
+ * workspace overwritten) and keep the fastest.  It does not change which form a plan's calls
+ * take (see cubic_rl_plan_variants): a plan in the fused form gains nothing from it.  Synchronises the stream several times, so
  * do not call it while capturing a graph.  The choice is remembered for later plans of
  * the same dims in this process and, if the environment variable CUBIC_TUNE_CACHE names a
  * file, appended there and read back by later processes. */

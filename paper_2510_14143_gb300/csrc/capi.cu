@@ -330,7 +330,7 @@ struct cubic_rl_plan_s {
     float *Hr = nullptr;        // [nz][ny][xp], owned
     // the fused form (plane.cuh): fuse.ok where it serves this plan; HF / HFr are H in its
     // layout (owned, or H itself where own_hf is false); pinned: the caller chose launch
-    // shapes or chunks of the pass-by-pass form, which plain calls then take
+    // shapes of the pass-by-pass form, which plain calls then take (as with column chunks)
     struct Fused {
         bool ok = false;
         PlaneGeo g;
@@ -342,7 +342,7 @@ struct cubic_rl_plan_s {
         bool c_is_z = false;
     } fuse;
     float2 *ftab = nullptr;           // the fused form's constants (plane_tables), owned
-    bool pinned = false;
+    bool pinned = false;  // by cubic_rl_plan_set_variants, for good
     float2 *HF = nullptr;
     float *HFr = nullptr;
     bool own_hf = false;
@@ -434,7 +434,7 @@ static const int kXKind[XM_COUNT] = {KK_X_FWD, KK_X_INV, KK_X_RATIO, KK_X_UPDATE
 
 // ------------------------------------------------------------------ the fused form
 
-static bool use_fused(const cubic_rl_plan_s *p) { return p->fuse.ok && !p->pinned; }
+static bool use_fused(const cubic_rl_plan_s *p) { return p->fuse.ok && !p->pinned && p->chunk == 0; }
 
 // Largest plane that takes the fused form
 constexpr int64_t kFuseSmem = 122 * 1024;
@@ -701,14 +701,16 @@ static cudaError_t run_conv(cubic_rl_plan_s *p, const ConvArgs &a, int zmode, cu
 // With p->chunk > 0 the three passes run chunk by chunk over groups of
 // p->chunk spectrum columns, so that a chunk written by one pass is still in
 // L2 when the next pass reads it: per voxel, HBM then sees one read and one
-// write of the spectrum (plus H) instead of three of each.
+// write of the spectrum (plus H) instead of three of each.  A chunk is rounded up to whole
+// tiles of the shapes in use (all powers of two): the tile pipelines start at tile boundaries.
 static cubic_status_t enqueue_yzy(cubic_rl_plan_s *p, float2 *spec, int zmode, cudaStream_t st)
 {
     if (use_fused(p)) {
         CUBIC_CUDA(run_conv(p, conv_args(p, spec), zmode, st));
         return CUBIC_OK;
     }
-    const int64_t step = p->chunk > 0 ? p->chunk : p->xh;
+    const int64_t tile = std::max(p->ky->yzv[p->vy].ycols, p->kz->yzv[p->vz].zcols);
+    const int64_t step = p->chunk > 0 ? (p->chunk + tile - 1) / tile * tile : p->xh;
     for (int64_t c0 = 0; c0 < p->xh; c0 += step) {
         const int64_t c1 = c0 + step < p->xh ? c0 + step : p->xh;
         CUBIC_CUDA(run_y(p, y_args(p, spec, 0, c0, c1), st));
@@ -1569,7 +1571,6 @@ extern "C" cubic_status_t cubic_rl_plan_set_chunk(cubic_rl_plan_t plan, int64_t 
     if (!plan) return fail(CUBIC_ERR_INVALID_ARG, "plan must be non-null");
     if (columns < 0 || columns % 16 != 0) return fail(CUBIC_ERR_INVALID_ARG, "chunk must be a multiple of 16 (0: off)");
     plan->chunk = columns;
-    if (columns > 0) plan->pinned = true;
     return CUBIC_OK;
 }
 

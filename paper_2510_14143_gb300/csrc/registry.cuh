@@ -39,6 +39,7 @@ struct XVariant {
 struct YZVariant {
     int P = 0, B = 0;
     bool tma = false;  // persistent TMA-pipelined kernel
+    int ycols = 1, zcols = 1;  // a launch over columns col0 .. col1 - 1 starts at a multiple of these
     YLaunch y = nullptr;
     ZLaunch z = nullptr;
     // plain variants: the same kernels over a table of volumes (null for TMA variants,
@@ -303,6 +304,8 @@ YZVariant make_yzvariant_tma()
     v.P = P;
     v.B = BY;
     v.tma = true;
+    if constexpr (BY > 0) v.ycols = BY;
+    if constexpr (BZ > 0) v.zcols = BZ;
     if constexpr (BY > 0)
         v.y = launch_y_tma<N, P, BY, NSY>;
     else
