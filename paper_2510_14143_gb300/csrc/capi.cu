@@ -343,6 +343,7 @@ struct cubic_rl_plan_s {
     } fuse;
     float2 *ftab = nullptr;           // the fused form's constants (plane_tables), owned
     bool pinned = false;  // by cubic_rl_plan_set_variants, for good
+    bool tuned = false;   // vx, vy, vz are measured, here or for another plan of these dims
     float2 *HF = nullptr;
     float *HFr = nullptr;
     bool own_hf = false;
@@ -851,12 +852,60 @@ static cubic_status_t rebuild_h(cubic_rl_plan_s *p, const float *psf, cudaStream
     return CUBIC_OK;
 }
 
+// The launch shapes of a plan that was not tuned; the Y pass of a large volume goes by the kind of
+// its PSF's spectrum
+static void default_variants(cubic_rl_plan_s *p)
+{
+    if (p->tuned || p->pinned) return;
+    const bool past_l2 = !p->linear && p->nz >= kPastL2Z && p->V * (int64_t)sizeof(float) > kPastL2Bytes;
+    p->vx = p->kx->dx;
+    // a linear plan's tiles leave the zero rows out of their copies (61x487x501 with a 25x33x33
+    // PSF, 20 iterations: 7.08 ms with the tile pipeline, 7.27 with the two-stage Y kernel)
+    p->vy = p->linear ? 0 : !past_l2 ? p->ky->dy : p->use_real_h ? p->ky->ly_real : p->ky->ly_cplx;
+    p->vz = p->kz->dz;
+    if (past_l2 && p->ky->yzv[p->vy].tma) p->vx = p->kx->lx;
+}
+
+// Transforms alone, with no product between their passes, run on the default shapes whatever the
+// volume's size, for as long as this lives (FSC of 100x768x512 571 us, 595 on the tile pipeline).
+struct TransformShapes {
+    cubic_rl_plan_s *p;
+    int vx, vy;
+    explicit TransformShapes(cubic_rl_plan_s *plan) : p(plan), vx(plan->vx), vy(plan->vy)
+    {
+        if (p->tuned || p->pinned || p->linear) return;
+        p->vx = p->kx->dx;
+        p->vy = p->ky->dy;
+    }
+    ~TransformShapes()
+    {
+        p->vx = vx;
+        p->vy = vy;
+    }
+    TransformShapes(const TransformShapes &) = delete;
+};
+
+// Calls whose X passes sum the likelihood or take accelerated steps run on AxisKernels::hx for
+// as long as this lives, where the plan would run on the default shape (also if tuning chose it:
+// it timed plain passes).
+struct HeavyX {
+    cubic_rl_plan_s *p;
+    int vx;
+    explicit HeavyX(cubic_rl_plan_s *plan) : p(plan), vx(plan->vx)
+    {
+        if (!p->pinned && vx == p->kx->dx) p->vx = p->kx->hx;
+    }
+    ~HeavyX() { p->vx = vx; }
+    HeavyX(const HeavyX &) = delete;
+};
+
 // Whether a batch graph multiplies by the real or the complex spectrum is fixed when it is
 // captured, so a change between the two is a new state of the plan.
 static cubic_status_t load_psf(cubic_rl_plan_s *p, const float *psf, cudaStream_t st)
 {
     const bool real = p->use_real_h;
     const cubic_status_t s = rebuild_h(p, psf, st);
+    default_variants(p);
     if (p->use_real_h != real) p->state = g_plan_state.fetch_add(1);
     return s;
 }
@@ -894,11 +943,7 @@ static void tune_load_locked()
 
 static void tuned_variants(cubic_rl_plan_s *p)
 {
-    p->vx = p->kx->dx;
-    // a linear plan's tiles leave the zero rows out of their copies (61x487x501 with a 25x33x33
-    // PSF, 20 iterations: 7.08 ms with the tile pipeline, 7.27 with the two-stage Y kernel)
-    p->vy = p->linear ? 0 : p->ky->dy;
-    p->vz = p->kz->dz;
+    default_variants(p);
     std::lock_guard<std::mutex> lk(g_tune_mu);
     tune_load_locked();
     for (const TuneEntry &e : g_tune)
@@ -907,6 +952,7 @@ static void tuned_variants(cubic_rl_plan_s *p)
             p->vx = e.vx;
             p->vy = e.vy;
             p->vz = e.vz;
+            p->tuned = true;
         }
 }
 
@@ -1679,6 +1725,7 @@ extern "C" cubic_status_t cubic_rl_autotune(cubic_rl_plan_t plan, const float *i
         if (ms < best) { best = ms; bz = v; }
     }
     plan->vz = bz;
+    plan->tuned = true;
     plan->prof = prof;
     if (s == CUBIC_OK) s = prepare();  // leave finite data behind
     if (s == CUBIC_OK && plan->linear) s = lin_crop(plan, out_w, out, st);
@@ -2370,6 +2417,7 @@ extern "C" cubic_status_t cubic_rl_deconvolve_accel(cubic_rl_plan_t plan, const 
     cubic_status_t s = ensure_workspace(p);
     if (s != CUBIC_OK) return s;
     if ((s = ensure_accel(p)) != CUBIC_OK) return s;
+    const HeavyX heavy(p);
     cudaStream_t st = (cudaStream_t)stream;
     const size_t vol = acc_vol_bytes(p) / sizeof(float);
     float *xc = p->acc, *xn = p->acc + vol, *y = p->acc + 2 * vol, *gc = p->acc + 3 * vol, *gn = p->acc + 4 * vol;
@@ -2609,6 +2657,7 @@ extern "C" cubic_status_t cubic_rl_deconvolve_monitor(cubic_rl_plan_t plan, cons
         p->mon = (float *)m;
         p->mon_cap = max_iter;
     }
+    const HeavyX heavy(p);
     float *dslots = p->mon, *nslots = dslots + f_d, *rpart = nslots + f_n, *mpart = rpart + f_r, *rec = mpart + f_r;
     float *kept_b = rec + f_rec, *kept_r = kept_b + f_lin / 2;
     cudaStream_t st = (cudaStream_t)stream;
@@ -2855,6 +2904,7 @@ static cubic_status_t enqueue_fsc(cubic_rl_plan_s *p, const float *a, const floa
                                   cudaStream_t st)
 {
     cubic_status_t s;
+    const TransformShapes shapes(p);
     if ((s = enqueue_forward3(p, a, p->ws, 1.f, st)) != CUBIC_OK) return s;
     if ((s = enqueue_forward3(p, b, p->ws2, 1.f, st)) != CUBIC_OK) return s;
     CUBIC_CUDA(cudaMemsetAsync(p->fsc_sums, 0, 6 * (size_t)n_shells * sizeof(float), st));

@@ -52,6 +52,10 @@ struct AxisKernels {
     int n = 0;
     int nx = 0, nyz = 0;  // number of X and Y/Z variants
     int dx = 0, dy = 0, dz = 0;  // the X, Y and Z variants of a plan that was not tuned
+    // its Y variants for volumes past L2 with a real and a complex PSF spectrum, and its X variant
+    // beside a tile-pipeline Y chosen there
+    int ly_real = 0, ly_cplx = 0, lx = 0;
+    int hx = 0;  // in dx's place in calls that sum the likelihood or take accelerated steps
     XVariant xv[kMaxVariants];
     YZVariant yzv[kMaxVariants];
     // multi-volume launches (batched path): X with xv[0]'s shape, Y/Z with P0 x 16 columns
@@ -514,12 +518,19 @@ AxisKernels make_axis()
         // to few CTAs per SM by its staged operand rows: both prefetched
         if constexpr (S::kAlt && N <= 1024) push_x(k, make_xvariant<N, P0, S::lines(P0, 128), true, true>());
     }
-    // The warp-per-line kernels, the default where they exist: at every one of these lengths
-    // they are as fast as the best of the shapes above, or faster
+    // The warp-per-line kernels, the default where they exist: within 2% of the best of the
+    // shapes above, or faster, by themselves.  At 512 a butterfly has 32 elements, and two calls
+    // take the first shape instead: those whose pointwise step holds more per element (logarithms
+    // and compensated sums, or the accelerated step's second array, of 64 elements a thread; us an
+    // iteration, warp kernel -> first shape: monitored 64x512x512 365 -> 299, 144x256x512 371 -> 325,
+    // 16x512x512 98 -> 96; accelerated 347 -> 314, 352 -> 349, 100 -> 95), and volumes past L2 beside a
+    // tile-pipeline Y pass, where the early operand prefetch competes with it (128x512x512 plain
+    // 533 -> 510, complex spectrum 558 -> 533; 100x768x512 684 -> 661).
     if constexpr (xwarp_has(N)) {
         k.dx = k.nx;
         push_x(k, make_xvariant_warp<N>());
     }
+    k.hx = k.lx = N == 512 ? 0 : k.dx;
     constexpr int XL = S::lines(P0, 128);
     k.xm[XM_FWD] = launch_x_multi<N, P0, XL, XM_FWD>;
     k.xm[XM_INV] = launch_x_multi<N, P0, XL, XM_INV>;
@@ -588,11 +599,21 @@ AxisKernels make_axis()
         }
         if constexpr (yline_has(N)) {
             if constexpr (yline_default(N)) k.dy = k.nyz;
+            k.ly_real = yline_large(N, true) ? k.dy : 0;
+            k.ly_cplx = yline_large(N, false) ? k.dy : 0;
             push_yz(k, make_yzvariant_yline<N, P0, B0>());
         }
     }
     return k;
 }
+
+// Volumes of more bytes than this (three quarters of L2: the spectrum is as large, and the
+// pointwise operands pass through beside it) take the defaults for volumes past L2.  The Y
+// kernels are level at 75 MB (384) and 67 MB (512) and 3 to 4% apart at 104 MB.
+constexpr int64_t kPastL2Bytes = 96 << 20;
+// ... if their Z pass is a tile pipeline too (lengths from 64).  Beside the plain Z kernels the
+// two-stage Y kernel stays ahead (48x768x1024: 645 us an iteration, 698 with the tile pipeline).
+constexpr int kPastL2Z = 64;
 
 // The supported lengths; shard s of the build instantiates entries i with
 // i % kShards == s.

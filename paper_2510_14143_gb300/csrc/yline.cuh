@@ -35,6 +35,17 @@ constexpr bool yline_has(int N) { return N >= 125 && yline_r0(N) > 1 && N / ylin
 // Whether a plan that was not tuned takes it: at 1024, where the tile pipeline has two 64 KB stages, a
 // volume larger than L2 is 20% slower with it (a smaller one 10% faster: the tuner's choice).
 constexpr bool yline_default(int N) { return yline_has(N) && N <= 768; }
+// The same for volumes past L2.  There the kernel's loads wait on HBM, and its advantage hangs on
+// what runs beside it.  Plain call, us an iteration, tile pipeline / this kernel, with a real PSF
+// spectrum: 384 (128 planes of 640 and 768, 100 of 1024) 504 / 537, 599 / 638, 624 / 675; 512 (128 of 512, 64 of
+// 1024, 81 of 768) 533 / 553, 525 / 554, 501 / 521; 768 (100 of 512 and 768, 64 of 768) 684 / 705, 998 /
+// 1051, 645 / 671.  With a complex one, which makes the Z pass the longer: 384 526 / 558, 627 / 668, 635 /
+// 622; 512 558 / 577, 548 / 544, 514 / 504; 768 694 / 656, 1023 / 980, 677 / 641.  256 and 640 gain in
+// either case (128 of 1024: 577 / 506; 90 of 768: 768 / 732).
+constexpr bool yline_large(int N, bool real_h)
+{
+    return yline_default(N) && N != 512 && !(real_h && (N == 384 || N == 768));
+}
 // columns per CTA: 128-byte segments where they leave room for two CTAs per SM
 constexpr int yline_cols(int N) { return N <= 320 || N == 512 ? 16 : 8; }
 // first-stage butterflies per thread: with R1 = 2 R0 two of them hold what the second stage's does
