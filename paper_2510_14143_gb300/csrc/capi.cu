@@ -2776,14 +2776,20 @@ constexpr int kFscMaxShells = 1024;
 
 // Shell sums in compensated float32: per thread over a run of kx, per block in shared memory,
 // then into the global pairs (value = hi + lo) -- sums[0..3S) high words, sums[3S..6S) low
-// words.  A thread takes kFscRun adjacent kx of one row: the shell only grows along them, so
+// words.  A thread takes RUN adjacent kx of one row: the shell only grows along them, so
 // one exact search serves the run and the shared-memory atomics are one set per shell crossed
 // instead of one per element, with the lanes of a warp in different shells.  Integers: with L
 // the dims' least common multiple, rho^2 = rn / L^2, rn = sum (k L / n)^2; Int is int64 where
 // 3 S^2 L^2 fits it.
-constexpr int kFscRun = 8;
+//
+// A run is a chain of dependent sums and atomics.  Runs of 8 (kFscRun) need enough of them to
+// hide it; volumes with fewer take runs of 2 (us a call, runs of 8 -> 2: 50x108x45 50.8 -> 33.5,
+// 48x90x40 75.4 -> 54.8, 15x36x32 57.4 -> 47.2, 27x81x128 42.7 -> 35.6, 20x96x192 37.5 -> 36.4).  Those
+// have fewer than 2^20 voxels, so their arithmetic fits int64 at any number of shells.
+constexpr int kFscRun = 8, kFscRunSmall = 2;
+constexpr int64_t kFscRuns = 152 * 256;  // a CTA per SM
 
-template <class Int>
+template <class Int, int RUN>
 __global__ void __launch_bounds__(256) k_fsc_bins(const float2 *__restrict__ A, const float2 *__restrict__ B,
                                                   int nz, int ny, int nx, int xh, int64_t xp, int64_t L, int S,
                                                   int copies, float *__restrict__ sums)
@@ -2796,19 +2802,19 @@ __global__ void __launch_bounds__(256) k_fsc_bins(const float2 *__restrict__ A, 
     const int64_t fz = L / nz, fy = L / ny, fx = L / nx;
     const Int den = (Int)L * L, S4 = (Int)4 * S * S;
     const float scale = 2.f * (float)S / (float)L;
-    const unsigned nruns = (unsigned)(xh + kFscRun - 1) / kFscRun;
+    const unsigned nruns = (unsigned)(xh + RUN - 1) / RUN;
     const int64_t n = (int64_t)nz * ny * nruns;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t row = i / nruns;
-        const int k0 = (int)(i - row * nruns) * kFscRun, z = (int)(row / ny), y = (int)(row - (int64_t)z * ny);
+        const int k0 = (int)(i - row * nruns) * RUN, z = (int)(row / ny), y = (int)(row - (int64_t)z * ny);
         const int64_t kz = (2 * z > nz ? z - nz : z) * fz, ky = (2 * y > ny ? y - ny : y) * fy;
         const int64_t rzy = kz * kz + ky * ky;
         // rows are 128-byte aligned and padded to 16 columns: the run loads whole
-        float2 a[kFscRun], b[kFscRun];
+        float2 a[RUN], b[RUN];
         const float4 *a4 = reinterpret_cast<const float4 *>(A + row * xp + k0);
         const float4 *b4 = reinterpret_cast<const float4 *>(B + row * xp + k0);
 #pragma unroll
-        for (int j = 0; j < kFscRun / 2; ++j) {
+        for (int j = 0; j < RUN / 2; ++j) {
             const float4 u = __ldg(a4 + j), v = __ldg(b4 + j);
             a[2 * j] = make_float2(u.x, u.y);
             a[2 * j + 1] = make_float2(u.z, u.w);
@@ -2835,7 +2841,7 @@ __global__ void __launch_bounds__(256) k_fsc_bins(const float2 *__restrict__ A, 
         Int next = (Int)(sh + 1) * (sh + 1) * den;
         bool any = false;
 #pragma unroll
-        for (int j = 0; j < kFscRun; ++j) {
+        for (int j = 0; j < RUN; ++j) {
             const int kx = k0 + j;
             if (kx >= xh) break;
             const int64_t x = (int64_t)kx * fx;
@@ -2910,10 +2916,15 @@ static cubic_status_t enqueue_fsc(cubic_rl_plan_s *p, const float *a, const floa
     CUBIC_CUDA(cudaMemsetAsync(p->fsc_sums, 0, 6 * (size_t)n_shells * sizeof(float), st));
     int64_t L = p->nx;
     for (int64_t d : {p->ny, p->nz}) L = L / std::gcd(L, d) * d;
-    const unsigned grid = grid_for(p->rows * ((p->xh + kFscRun - 1) / kFscRun), 256, 152 * 4);
+    const bool small = p->rows * ((p->xh + kFscRun - 1) / kFscRun) < kFscRuns;
+    const int run = small ? kFscRunSmall : kFscRun;
+    const unsigned grid = grid_for(p->rows * ((p->xh + run - 1) / run), 256, 152 * 4);
     const int set = 6 * n_shells * (int)sizeof(float);
     const int copies = std::max(1, std::min(8, 40 * 1024 / set));  // of the block's sums
-    auto bins = 3.0 * n_shells * n_shells * (double)L * (double)L < 9e18 ? k_fsc_bins<int64_t> : k_fsc_bins<__int128>;
+    const bool fits = 3.0 * n_shells * n_shells * (double)L * (double)L < 9e18;
+    auto bins = small  ? k_fsc_bins<int64_t, kFscRunSmall>
+                : fits ? k_fsc_bins<int64_t, kFscRun>
+                       : k_fsc_bins<__int128, kFscRun>;
     bins<<<grid, 256, copies * set, st>>>(p->ws, p->ws2, (int)p->nz, (int)p->ny, (int)p->nx, (int)p->xh, p->xp, L, n_shells,
                                           copies, p->fsc_sums);
     k_fsc_final<<<(n_shells + 255) / 256, 256, 0, st>>>(p->fsc_sums, n_shells, fsc);
