@@ -469,7 +469,7 @@ static bool fuse_geometry(const cubic_rl_plan_s *p, bool c_is_z, cubic_rl_plan_s
     g.off_twc = (x.tw + 1) / 2 * 2;
     g.off_tab = g.off_twc + (c.tw + 1) / 2 * 2;
     g.off_neg = g.off_tab + (g.lines + 3) / 4 * 2;
-    g.off_plane = g.off_neg + (g.nc + 3) / 4 * 2;
+    g.off_plane = g.off_neg + (g.nc + 3) / 4 * 2 + 2;
     const int last = (g.nc + 1) / 2 - 1;  // pair lines 0 .. last
     const int64_t slots = (int64_t)(last / c.r1) * g.bs + (int64_t)(last % c.r1 + 1) * g.xs;
     const int64_t smem = ((int64_t)g.off_plane + slots) * (int64_t)sizeof(float2);

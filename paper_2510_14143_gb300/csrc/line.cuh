@@ -113,10 +113,10 @@ struct PointSums {
 };
 
 // The pointwise step: v[i].x is element o0 + P i of the real volumes, v[i].y element o1 + P i
-// (two: that row exists).
+// (two: that row exists).  center: the pair at XArgs::center, in shared memory (null: none).
 template <int MODE, int E, int P, class Off>
 __device__ __forceinline__ void plane_point(const XArgs &a, float2 (&v)[E], const Off o0, const Off o1,
-                                            const bool two, PointSums &sum)
+                                            const bool two, PointSums &sum, const float2 *center)
 {
     if constexpr (MODE == XM_FWD) {
         const float *s0 = a.src + o0, *s1 = a.src + o1;
@@ -176,8 +176,8 @@ __device__ __forceinline__ void plane_point(const XArgs &a, float2 (&v)[E], cons
             const float x1 = __fdividef(two ? __ldg(p1 + n) : 0.f, fmaxf(v[i].y, eps));
             v[i] = make_float2(x0, x1);
         });
-        if (a.center) {
-            const float c = __ldg(&a.center->x);
+        if (center) {
+            const float c = center->x;
             static_for<0, E>([&](auto i_) {
                 constexpr int i = CUBIC_CI(i_);
                 v[i] = make_float2(v[i].x - c, two ? v[i].y - c : 0.f);
@@ -193,8 +193,8 @@ __device__ __forceinline__ void plane_point(const XArgs &a, float2 (&v)[E], cons
     } else if constexpr (MODE == XM_UPDATE || MODE == XM_FINAL) {
         float *ob = (MODE == XM_FINAL || a.dst) ? a.dst : a.u;
         const float *p0 = a.u + o0, *p1 = a.u + o1;
-        if (a.center) {
-            const float h = __ldg(&a.center->y);
+        if (center) {
+            const float h = center->y;
             static_for<0, E>([&](auto i_) { v[CUBIC_CI(i_)] = cadd(v[CUBIC_CI(i_)], make_float2(h, h)); });
         }
         if (a.keep_a) {

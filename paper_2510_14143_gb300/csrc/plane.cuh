@@ -62,8 +62,9 @@ struct PlaneGeo {
     int nx = 0, nc = 0, np = 0;   // x, in-plane second axis, planes (the p axis)
     int lines = 0;                // c lines: nx / 2 (even nx, line 0 carries k = 0 and nx / 2), or (nx + 1) / 2
     int xs = 0, bs = 0, cr1 = 0;  // pitch of a pair line, of cr1 = R1 pair lines (complex slots)
-    // shared memory, in float2: [x twiddles][c twiddles][line slots][partners][plane]; what
-    // stands before the plane is copied from the plan's constant block
+    // shared memory, in float2: [x twiddles][c twiddles][line slots][partners][center][plane];
+    // what stands before the plane is copied from the plan's constant block, but for the center
+    // (2 float2, one used)
     int off_twc = 0, off_tab = 0, off_neg = 0, off_plane = 0;
     int smem = 0;                 // bytes
     int mv = 0, m = 0;            // a plane's spectrum: values, and pitch (a multiple of 16)
@@ -298,7 +299,7 @@ __device__ __forceinline__ void plane_col_forward(const PlaneGeo &g, float2 *__r
 // memory (false: the step starts from zeros, XM_ADJ_U); back: transform the result.
 template <int NX, int MODE>
 __device__ __forceinline__ void plane_rows(const PlaneArgs &a, float2 *plane, const float2 *twx, const int p,
-                                           const bool spec, const bool back, PointSums &sum)
+                                           const bool spec, const bool back, PointSums &sum, const float2 *center)
 {
     using F = Line<NX>;
     constexpr int R0 = F::R0, R1 = F::R1, Lw = row_lines(NX);
@@ -338,7 +339,7 @@ __device__ __forceinline__ void plane_rows(const PlaneArgs &a, float2 *plane, co
             }
             const int o = off + (m0 + l) * rs + j;
             // the last line of an odd nc has one row
-            plane_point<MODE, R0, R1>(a.x, x, o, o + second, m0 + l + H < a.g.nc, sum);
+            plane_point<MODE, R0, R1>(a.x, x, o, o + second, m0 + l + H < a.g.nc, sum, center);
             if (MODE != XM_INV && MODE != XM_FINAL && back) {
                 F::fwd0(x, twx, j);
                 static_for<0, R0>([&](auto r_) { q[CUBIC_CI(r_) * F::kStep] = x[CUBIC_CI(r_)]; });
@@ -459,6 +460,14 @@ __device__ __forceinline__ void plane_tables(const PlaneGeo &g, float2 *tab, con
 
 // ------------------------------------------------------------------ kernels
 
+// 8 bytes from global to shared memory, asynchronously; and the wait for this thread's copies
+__device__ __forceinline__ void copy_async8(void *dst, const void *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void copy_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 template <int MODE>
 __global__ void __launch_bounds__(kPlaneThreads, 1)
     k_plane(const __grid_constant__ PlaneArgs one, const PlaneTable *__restrict__ tab)
@@ -478,6 +487,8 @@ __global__ void __launch_bounds__(kPlaneThreads, 1)
     const uint32_t *neg = reinterpret_cast<const uint32_t *>(smem_pl + g.off_neg);
     float2 *plane = smem_pl + g.off_plane;
     constexpr bool kIn = MODE != XM_FWD, kOut = MODE != XM_INV && MODE != XM_FINAL;
+    constexpr bool kCenter = MODE == XM_RATIO || MODE == XM_UPDATE || MODE == XM_FINAL;
+    float2 *center = kCenter && a.x.center ? plane - 2 : nullptr;
 
     // constants of the plan: before the wait
     for (int i = threadIdx.x; i < g.off_plane / 2; i += blockDim.x)
@@ -492,6 +503,9 @@ __global__ void __launch_bounds__(kPlaneThreads, 1)
     }
     __syncthreads();
     pdl_wait();
+    // the center on its way under the loads of the spectrum, in shared memory and not in a register:
+    // loaded where it is used it cost 0.5 us a launch
+    if (kCenter && center && threadIdx.x == 0) copy_async8(center, a.x.center);
 
     const bool spec = kIn && (MODE != XM_ADJ_U || a.x.spec_in != nullptr);
     const bool back = kOut && (MODE != XM_ADJ_U || a.x.adj_u != nullptr);
@@ -499,6 +513,7 @@ __global__ void __launch_bounds__(kPlaneThreads, 1)
         if (spec) {
             len_switch(PlaneC{}, g.nc,
                        [&](auto n_) { plane_col_inverse<CUBIC_CI(n_)>(g, a.x.spec_in + p * g.m, plane, twc, slots); });
+            if (kCenter) copy_async_wait();
             __syncthreads();
         }
     }
@@ -507,7 +522,7 @@ __global__ void __launch_bounds__(kPlaneThreads, 1)
     // (128x64x128 voxels, 256 threads: 43.9 us an iteration, 28.2 us with the release here).
     pdl_trigger();
     PointSums sum;
-    len_switch(PlaneX{}, g.nx, [&](auto n_) { plane_rows<CUBIC_CI(n_), MODE>(a, plane, twx, p, spec, back, sum); });
+    len_switch(PlaneX{}, g.nx, [&](auto n_) { plane_rows<CUBIC_CI(n_), MODE>(a, plane, twx, p, spec, back, sum, center); });
     if constexpr (kOut) {
         if (back) {
             __syncthreads();
