@@ -340,6 +340,7 @@ struct cubic_rl_plan_s {
         size_t tab_elems = 0;         // the constant block, float2
         size_t off_center = 0;        // in it: the ratio's centre, then kReduceBlocks counts
         bool c_is_z = false;
+        double us = 0.0;              // what an iteration is expected to take (fuse_geometry)
     } fuse;
     float2 *ftab = nullptr;           // the fused form's constants (plane_tables), owned
     bool pinned = false;  // by cubic_rl_plan_set_variants, for good
@@ -505,6 +506,13 @@ static bool fuse_geometry(const cubic_rl_plan_s *p, bool c_is_z, cubic_rl_plan_s
         }
     }
     f->threads = 32 * best;
+    // An iteration's time by what its longest warp does: two plane launches of best_cost (6% more
+    // where an odd c takes its extra passes), two convolution launches, whose warps fill the SMs to
+    // 28, and the launches themselves.  Fitted over 119 volumes (9x144x144 to 160x192x144) and both
+    // choices of c, 190 times in all: 7.6% rms.
+    const double conv = task_cost(v, v.conv_lines);
+    f->us = 13.8 + 0.158 * (double)best_cost * (g.nc % 2 ? 1.06 : 1.0) + 0.134 * conv +
+            1.276 * conv * (double)g.mv / (v.conv_lines * 152.0 * 28.0);
     return true;
 }
 
@@ -516,10 +524,16 @@ static void fuse_setup(cubic_rl_plan_s *p)
     const bool hz = fuse_geometry(p, true, &z), hy = fuse_geometry(p, false, &y);
     // the smaller plane (more CTAs, and more of them on an SM), but an even c axis before an odd
     // one, which takes two more passes over the plane (81x150x135 voxels: 69 us an iteration
-    // with c = 150, 87 us with c = 81)
+    // with c = 150, 87 us with c = 81); against this where the other choice should be faster by
+    // more than 5% (45x100x192, where c = 100 leaves 45 planes for 152 SMs: 52 us an iteration, 44
+    // with c = 45; 160x150x120 84 -> 69; 96x160x108 62 -> 58; 90x150x90 60 -> 54; over 119 volumes none
+    // measured slower)
     auto cost = [](const cubic_rl_plan_s::Fused &f) { return f.g.nc + (f.g.nc % 2 ? 1024 : 0); };
-    if (hz && (!hy || cost(z) <= cost(y))) p->fuse = z;
-    else if (hy) p->fuse = y;
+    const bool by_z = hz && (!hy || cost(z) <= cost(y));
+    if (hz && hy)
+        p->fuse = by_z ? (y.us < 0.95 * z.us ? y : z) : (z.us < 0.95 * y.us ? z : y);
+    else if (hz || hy)
+        p->fuse = hz ? z : y;
 }
 
 // the plan's constant block, from its twiddle tables
