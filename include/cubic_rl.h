@@ -114,6 +114,7 @@ CUBIC_API cubic_status_t cubic_rl_deconvolve(cubic_rl_plan_t plan, const float *
  * serves one volume).  images[v], outs[v]: device float32 volumes of plans[v]'s dims.  Small
  * and medium volumes (axes of at most 192, an (x, y) or (x, z) plane of at most 122 KB) take the
  * fused form, one plane kernel and one convolution kernel per half iteration over all of them;
+ * other volumes of at least 4 million voxels run the plain call's passes one after the other;
  * the volumes of any other size share one launch per pass and
  * length, whose launch shape (threads per line, lines or columns per CTA) is tuned the first
  * time the length appears: every candidate is timed on the call's own buffers and the
@@ -121,8 +122,8 @@ CUBIC_API cubic_status_t cubic_rl_deconvolve(cubic_rl_plan_t plan, const float *
  * n_iter sequence is captured once into a CUDA graph (first call with a given argument
  * set: tuning of new lengths, capture and instantiation, synchronous) and replayed on
  * `stream` by later calls with identical arguments (a few argument sets are cached).  A plan
- * that got another workspace or wait limit since, or whose PSF changed between symmetric and
- * not, has its sequence captured anew; destroying a plan drops the graphs that run it.
+ * that got another workspace, wait limit, launch shape or chunk since, or whose PSF changed between
+ * symmetric and not, has its sequence captured anew; destroying a plan drops the graphs that run it.
  * 1 <= n <= 256.  Errors: INVALID_ARG, ALIGNMENT, OUT_OF_MEMORY, CUDA. */
 CUBIC_API cubic_status_t cubic_rl_deconvolve_batched(const cubic_rl_plan_t *plans, int n,
                                                      const float *const *images, int n_iter, float eps,

@@ -292,8 +292,8 @@ static std::atomic<uint64_t> g_plan_state{1};
 
 struct cubic_rl_plan_s {
     int device = 0;
-    // renewed whenever something that the batched path's tables hold changes: work array, kind
-    // and buffers of H, wait limit
+    // renewed whenever something that the batched path's tables and captured launches hold
+    // changes: work array, kind and buffers of H, wait limit, launch shapes and chunks
     uint64_t state = g_plan_state.fetch_add(1);
     int64_t nz = 0, ny = 0, nx = 0, V = 0, rows = 0, xh = 0, xp = 0;
     const AxisKernels *kx = nullptr, *ky = nullptr, *kz = nullptr;
@@ -1623,6 +1623,7 @@ extern "C" cubic_status_t cubic_rl_plan_set_variants(cubic_rl_plan_t plan, int v
     plan->vy = vy;
     plan->vz = vz;
     plan->pinned = true;
+    plan->state = g_plan_state.fetch_add(1);
     return CUBIC_OK;
 }
 
@@ -1631,6 +1632,7 @@ extern "C" cubic_status_t cubic_rl_plan_set_chunk(cubic_rl_plan_t plan, int64_t 
     if (!plan) return fail(CUBIC_ERR_INVALID_ARG, "plan must be non-null");
     if (columns < 0 || columns % 16 != 0) return fail(CUBIC_ERR_INVALID_ARG, "chunk must be a multiple of 16 (0: off)");
     plan->chunk = columns;
+    plan->state = g_plan_state.fetch_add(1);
     return CUBIC_OK;
 }
 
@@ -1740,6 +1742,7 @@ extern "C" cubic_status_t cubic_rl_autotune(cubic_rl_plan_t plan, const float *i
     }
     plan->vz = bz;
     plan->tuned = true;
+    plan->state = g_plan_state.fetch_add(1);
     plan->prof = prof;
     if (s == CUBIC_OK) s = prepare();  // leave finite data behind
     if (s == CUBIC_OK && plan->linear) s = lin_crop(plan, out_w, out, st);
@@ -3012,7 +3015,8 @@ extern "C" cubic_status_t cubic_fsc_split(cubic_rl_plan_t half_plan, const float
 //
 // Many volumes of different sizes in one CUDA graph.  The volumes that the fused form serves
 // share its launches: the planes of all volumes of one size group in one launch per half
-// iteration, the p-axis convolutions of all of them in another.  The others share one launch
+// iteration, the p-axis convolutions of all of them in another.  Large volumes run the plain
+// call's passes.  The others share one launch
 // per pass and axis length (k_*pass with a MultiTable).  A launch's blocks are the
 // concatenation of every member volume's blocks, and each block finds its volume in a
 // device-side table.  The whole n_iter sequence is captured once into a graph and replayed on
@@ -3067,6 +3071,7 @@ struct BatchState {
     std::vector<ZGroup> gz;
     std::vector<PlaneGroup> fp;
     std::vector<ConvGroup> fc;
+    std::vector<int> alone;  // volumes that run the plain call's passes
     void *dmem = nullptr;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
@@ -3102,11 +3107,13 @@ static void drop_batches(const cubic_rl_plan_s *p)
 
 static cubic_status_t enqueue_batched(BatchState &b, cudaStream_t st)
 {
-    for (size_t v = 0; v < b.plans.size(); ++v) {
-        cubic_status_t s = enqueue_init(b.plans[v], b.images[v], b.eps, b.outs[v], st);
+    for (int v = 0; v < (int)b.plans.size(); ++v) {
+        const bool alone = std::find(b.alone.begin(), b.alone.end(), v) != b.alone.end();
+        cubic_status_t s = alone ? enqueue_rl(b.plans[v], b.images[v], b.n_iter, b.eps, b.outs[v], b.plans[v]->ws, st)
+                                 : enqueue_init(b.plans[v], b.images[v], b.eps, b.outs[v], st);
         if (s != CUBIC_OK) return s;
     }
-    if (b.n_iter == 0) return CUBIC_OK;
+    if (b.n_iter == 0 || b.alone.size() == b.plans.size()) return CUBIC_OK;
     auto xstage = [&](int mode) -> cubic_status_t {
         for (const PlaneGroup &g : b.fp)
             CUBIC_CUDA(launch_plane(mode, PlaneArgs{}, g.tab, g.blocks, g.threads, g.smem, st));
@@ -3361,6 +3368,14 @@ static cubic_status_t batch_tune(BatchState &b, const LenGroups &byx, const LenG
 
 // Group volumes by axis length, tune the launch shapes of new lengths, and build the
 // device tables.
+// Volumes of this many voxels outside the fused form fill the GPU by themselves: they run the
+// plain call's passes one volume after the other.  Those have kernels that the launches over
+// tables of volumes lack (tile pipelines, warp-per-line X, two-stage Y).  10 iterations, us, shared launches -> one by
+// one: 2 of 128x256x256 3459 -> 2161, 4 of 64x256x256 3353 -> 2490, 3 of 100x160x256 2365 -> 1909, 2 of
+// 144x160x256 2102 -> 1696.  Below the line it goes either way (4 of 48x256x256 2308 -> 2109, 3 of 80x256x192
+// 2254 -> 2434, 8 of 64x128x256 3210 -> 3577, 6 of 16x256x512 2439 -> 3061).
+constexpr int64_t kAloneVoxels = 4000000;
+
 static cubic_status_t build_batch(BatchState &b, cudaStream_t st)
 {
     const int n = (int)b.plans.size();
@@ -3374,6 +3389,10 @@ static cubic_status_t build_batch(BatchState &b, cudaStream_t st)
             while (p->fuse.g.smem > kGroupSmem[i]) ++i;
             planes[i].push_back(v);
             convs.push_back(v);
+            continue;
+        }
+        if (p->V >= kAloneVoxels) {
+            b.alone.push_back(v);
             continue;
         }
         byx[p->nx].push_back(v);
@@ -3390,6 +3409,7 @@ static cubic_status_t build_batch(BatchState &b, cudaStream_t st)
                                  sizeof(MultiTable<XArgs>), sizeof(MultiTable<YArgs>), sizeof(MultiTable<ZArgs>)});
     const size_t stride = (tsz + 255) / 256 * 256;
     std::vector<unsigned char> host(stride * ntab, 0);
+    if (ntab == 0) return CUBIC_OK;
     CUBIC_CUDA(cudaMalloc(&b.dmem, host.size()));
     unsigned char *dbase = (unsigned char *)b.dmem;
     size_t slot = 0;
