@@ -524,14 +524,17 @@ static void fuse_setup(cubic_rl_plan_s *p)
     const bool hz = fuse_geometry(p, true, &z), hy = fuse_geometry(p, false, &y);
     // the smaller plane (more CTAs, and more of them on an SM), but an even c axis before an odd
     // one, which takes two more passes over the plane (81x150x135 voxels: 69 us an iteration
-    // with c = 150, 87 us with c = 81); against this where the other choice should be faster by
-    // more than 5% (45x100x192, where c = 100 leaves 45 planes for 152 SMs: 52 us an iteration, 44
-    // with c = 45; 160x150x120 84 -> 69; 96x160x108 62 -> 58; 90x150x90 60 -> 54; over 119 volumes none
-    // measured slower)
+    // with c = 150, 87 us with c = 81); against this where the first choice has planes for at
+    // most a third of the SMs and the other should be faster by more than 5% (45x100x192, where
+    // c = 100 leaves 45 planes for 152 SMs: 52 us an iteration, 44 with c = 45; 45x60x192 46 -> 40).
+    // With more planes the smaller ones share SMs with other volumes of a batch or other streams,
+    // which the estimate does not see (16 differentiable 64x128x128 volumes over 4 streams: 34 ms
+    // with c = 64, 38 with the c = 128 that it prefers)
     auto cost = [](const cubic_rl_plan_s::Fused &f) { return f.g.nc + (f.g.nc % 2 ? 1024 : 0); };
     const bool by_z = hz && (!hy || cost(z) <= cost(y));
+    const cubic_rl_plan_s::Fused &first = by_z ? z : y, &other = by_z ? y : z;
     if (hz && hy)
-        p->fuse = by_z ? (y.us < 0.95 * z.us ? y : z) : (z.us < 0.95 * y.us ? z : y);
+        p->fuse = 3 * first.g.np <= 152 && other.us < 0.95 * first.us ? other : first;
     else if (hz || hy)
         p->fuse = hz ? z : y;
 }
@@ -3016,8 +3019,8 @@ extern "C" cubic_status_t cubic_fsc_split(cubic_rl_plan_t half_plan, const float
 // Many volumes of different sizes in one CUDA graph.  The volumes that the fused form serves
 // share its launches: the planes of all volumes of one size group in one launch per half
 // iteration, the p-axis convolutions of all of them in another.  Large volumes run the plain
-// call's passes.  The others share one launch
-// per pass and axis length (k_*pass with a MultiTable).  A launch's blocks are the
+// call's passes.  The others share one launch per pass and axis length (k_*pass with a
+// MultiTable).  A launch's blocks are the
 // concatenation of every member volume's blocks, and each block finds its volume in a
 // device-side table.  The whole n_iter sequence is captured once into a graph and replayed on
 // later calls with the same arguments.
@@ -3366,8 +3369,6 @@ static cubic_status_t batch_tune(BatchState &b, const LenGroups &byx, const LenG
     return s;
 }
 
-// Group volumes by axis length, tune the launch shapes of new lengths, and build the
-// device tables.
 // Volumes of this many voxels outside the fused form fill the GPU by themselves: they run the
 // plain call's passes one volume after the other.  Those have kernels that the launches over
 // tables of volumes lack (tile pipelines, warp-per-line X, two-stage Y).  10 iterations, us, shared launches -> one by
@@ -3376,6 +3377,8 @@ static cubic_status_t batch_tune(BatchState &b, const LenGroups &byx, const LenG
 // 2254 -> 2434, 8 of 64x128x256 3210 -> 3577, 6 of 16x256x512 2439 -> 3061).
 constexpr int64_t kAloneVoxels = 4000000;
 
+// Group volumes by axis length, tune the launch shapes of new lengths, and build the
+// device tables.
 static cubic_status_t build_batch(BatchState &b, cudaStream_t st)
 {
     const int n = (int)b.plans.size();

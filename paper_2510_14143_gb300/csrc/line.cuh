@@ -35,7 +35,6 @@ constexpr int plane_r0(int N)
     return best;
 }
 constexpr int plane_r1(int N) { return N / plane_r0(N); }
-constexpr int plane_max_radix(int N) { return plane_r0(N) > plane_r1(N) ? plane_r0(N) : plane_r1(N); }
 
 // Share of the lanes that work when a warp runs w lines of length N, both stages weighted by
 // their elements, in percent
@@ -113,7 +112,9 @@ struct PointSums {
 };
 
 // The pointwise step: v[i].x is element o0 + P i of the real volumes, v[i].y element o1 + P i
-// (two: that row exists).  center: the pair at XArgs::center, in shared memory (null: none).
+// (two: that row exists).  center: the pair at XArgs::center, or a
+// copy of it in shared memory (null: none; k_xwarp passes the argument's, always null there, and
+// not a literal: without the branches the ratio kernel at 256 measured 10% slower).
 template <int MODE, int E, int P, class Off>
 __device__ __forceinline__ void plane_point(const XArgs &a, float2 (&v)[E], const Off o0, const Off o1,
                                             const bool two, PointSums &sum, const float2 *center)

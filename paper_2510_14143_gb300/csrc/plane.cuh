@@ -6,12 +6,13 @@
 // and runs, in one kernel, the inverse c transform, the inverse x transform, the pointwise
 // Richardson-Lucy step, the forward x transform and the forward c transform (k_plane).  A
 // second kernel (k_conv) does the p axis: forward transform, product with H, inverse
-// transform.  An iteration is then 4 launches instead of 8 and moves 48 bytes per voxel
-// instead of 84 (a spectrum in and one out per kernel, H, and the pointwise operands).
+// transform.  An iteration is then 4 launches instead of 8 and moves 52 bytes per voxel
+// instead of 84 (a spectrum in and one out per kernel, H, and the pointwise operands), or 48
+// instead of 80 with a real H.
 //
 // At these sizes a kernel visits its code once or twice, so instruction fetch (32 KB of
 // first-level instruction cache) and latency bound it before anything else.  Hence:
-//   - Every length is a product of two radices, N = R0 R1 (at most 16 each up to 256), and a
+//   - Every length is a product of two radices, N = R0 R1 (at most 16 each, but 125 = 5 x 25), and a
 //     stage is a rolled loop over one radix butterfly per thread.  The loops' bodies are all
 //     the code there is, and no thread holds more than one butterfly.
 //   - Transforms are in place: decimation in frequency forward, decimation in time back, so
@@ -20,7 +21,8 @@
 //     read, so an exchange needs one synchronisation instead of two; a convolution never
 //     needs the natural order.
 //   - The lines of a task belong to ONE warp: exchanges synchronise the warp, not the CTA.
-//     A plane kernel has two CTA barriers in all (between its c and x parts).
+//     A plane kernel has three CTA barriers: after its constants are copied, and between its c
+//     and x parts (accelerated runs add two for their sums).
 //   - Rows c and c + nc/2 share one complex line, z = row_c + i row_(c+nc/2).  Splitting
 //     Z[k], Z[nx-k] into the two rows' spectra happens where the c transform loads them: the
 //     thread that holds element c of frequency line k also holds element c + nc/2, so the

@@ -2,8 +2,8 @@
 // there are one or more compiled launch-shape variants of each pass:
 //   X pass: threads per line P and line pairs per CTA L (all five modes)
 //   Y / Z pass: threads per line P and adjacent columns per CTA B
-// Variant 0 is the default; the autotuner (tuner.cu) times the others on a
-// plan's own buffers and picks per pass.
+// AxisKernels::dx, dy and dz are the defaults; the autotuner (cubic_rl_autotune) times
+// all of them on a plan's own buffers and picks per pass.
 #pragma once
 
 #include <cuda_runtime.h>

@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(kXWarps * 32, (N <= 256 ? 3 : 2)) k_xwarp(cons
         }
         if (!kIn) static_for<0, R0>([&](auto r_) { x[CUBIC_CI(r_)] = make_float2(0.f, 0.f); });
         const int64_t o = 2 * pair * N + j;
-        if (pair < pairs) plane_point<MODE, R0, R1>(a, x, o, o + N, 2 * pair + 1 < a.rows, sum, nullptr);
+        if (pair < pairs) plane_point<MODE, R0, R1>(a, x, o, o + N, 2 * pair + 1 < a.rows, sum, a.center);
         if constexpr (kOut) {
             F::fwd0(x, tw, j);
             static_for<0, R0>([&](auto r_) { q[CUBIC_CI(r_) * F::kStep] = x[CUBIC_CI(r_)]; });

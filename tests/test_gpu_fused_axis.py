@@ -25,7 +25,7 @@ def dev(a):
     return torch.from_numpy(np.ascontiguousarray(a, dtype=np.float32)).cuda()
 
 
-# the first two leave the even axis, the third the smaller plane; the others keep it
+# the first two leave the even axis for the odd one, the last one the smaller plane
 @pytest.mark.parametrize("shape", [(45, 100, 192), (45, 60, 192), (54, 64, 90), (75, 80, 144), (45, 64, 64), (45, 75, 81), (18, 32, 54)])
 def test_convolve(cr, shape):
     r = np.random.default_rng(sum(shape))
